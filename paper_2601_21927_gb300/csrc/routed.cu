@@ -4,7 +4,8 @@
 // buffers of their own, each at the row itself or at a caller-given row (so
 // the K and V of new tokens land straight in their retained-cache rows).
 //
-// Launches, none of which needs a host round trip:
+// At most 192 rows take one kernel, routed_small (see there).  More take four
+// launches, none of which needs a host round trip:
 //   role_count    per 1024-row chunk: its Nexus rows;
 //   role_order    per chunk: the stable partition [ordinary rows | Nexus rows]
 //                 (perm[g] = source row of grouped row g) and the two group
@@ -16,6 +17,8 @@
 //                 output tiles of the grouped rows.  A tile never straddles
 //                 the two groups, so each tile reads one weight matrix; the
 //                 epilogue writes bf16 rows to the parts.
+#include <atomic>
+
 #include "sonic_dev.cuh"
 #include "sonic_host.h"
 
@@ -214,24 +217,6 @@ __device__ __forceinline__ GemmTile gemm_tile(int i, int n0, int n1, int mt0, in
 constexpr uint64_t kCopyGraceNs = 200000;
 
 // ---- CTA-pair primitives (clusters of two CTAs; rank 0 leads)
-
-__device__ __forceinline__ uint32_t cluster_rank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-
-// Address of the same shared-memory offset in CTA `rank` of the cluster.
-__device__ __forceinline__ uint32_t smem_in_rank(const void *p, uint32_t rank) {
-    uint32_t a;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
-    return a;
-}
-
-__device__ __forceinline__ void cluster_sync_all() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\t"
-                 "barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
 
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr)
@@ -483,6 +468,280 @@ routed_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
     if (warp == 1) tmem_dealloc_pair(tmem, 512);
 }
 
+// ------------------------------------------------------------- few rows
+//
+// T <= 192 rows: a generation step's projections, or a short turn's.  The call is
+// bound by streaming the weights (4096 -> 6144: 50 MB), so the weights are the M
+// operand: a cluster of S CTAs takes 128 weight rows, each CTA a share of the
+// reduction, and NT >= T rows of X (unordered: no partition, no copy) are the N
+// operand.  S is the largest that keeps all clusters resident at once, so nearly
+// every SM streams its own share of the weights and no tile waits for a second
+// wave.  Both weight matrices are streamed where the rows hold both kinds, each
+// into an accumulator of its own, and the epilogue picks by role; with one kind
+// only, the other matrix is not read.  The partial sums (fp32) meet through
+// distributed shared memory in rank order.
+// The 256 x 256 pair tiles that larger calls take keep 48 of 152 SMs busy here,
+// behind three more kernels.  GPU time of 4096 -> 6144 in us, those / this:
+// 28.8 / 15.1 at 16 rows (of it ~5 before the first and after the last copy, the
+// weights at 5 TB/s in between), 30.9 / 16.8 at 64, 31.8 / 19.6 at 128 (the N
+// operand now as large as the weights' share), 32.5 / 25.6 at 64 with both kinds.
+// The line lies at 192 rows because a CTA reads all of X per weight tile: at 256
+// rows it was 32.2 / 28.3 with one kind and 37.7 / 40.8 with both.  Two CTAs per
+// SM with half the ring each were no faster (15.5 at 16 rows, 23.1 at 128).
+
+template <int NT>
+struct SmallCfg {
+    static constexpr int kWBytes = kHalfN * kGBK * 2;  // 16 KB: 128 weight rows
+    static constexpr int kXBytes = NT * kGBK * 2;
+    static constexpr int kStageBytes = kWBytes + kXBytes;
+    static constexpr int kStages = NT <= 32 ? 10 : (192 * 1024) / kStageBytes;
+    static constexpr int kRing = kStages * kStageBytes;
+    static constexpr int kPartBytes = NT * kHalfN * 4;  // partial sums, over the ring
+    static_assert(kPartBytes <= kRing, "partial sums fit the ring");
+    static constexpr int kOffBar = kRing;
+    static constexpr int kNumBars = 2 * kStages + 1;
+    static constexpr int kOffMisc = kOffBar + kNumBars * 8;
+    static constexpr size_t kSmem = 1024 + kOffMisc + 64;
+    // two accumulators, a power of two
+    static constexpr uint32_t kTmemCols = NT <= 16 ? 32 : NT <= 32 ? 64 : NT <= 64 ? 128
+                                          : NT <= 128 ? 256 : 512;
+};
+
+constexpr int kSmallRows = 192;
+
+template <int NT>
+__global__ void __launch_bounds__(kGThreads, 1)
+routed_small_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW,
+                    const __grid_constant__ CUtensorMap tmWn, const uint8_t *role,
+                    const GemmParams p, int n_split) {
+    using C = SmallCfg<NT>;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *smem = reinterpret_cast<uint8_t *>(
+        (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+    uint64_t *full = reinterpret_cast<uint64_t *>(smem + C::kOffBar);
+    uint64_t *empty = full + C::kStages;
+    uint64_t *acc_full = empty + C::kStages;
+    int32_t *misc = reinterpret_cast<int32_t *>(smem + C::kOffMisc);
+    // misc: 0 tensor memory, 1 abort, 2 kinds of rows, 4-9 Nexus bits of the rows
+    volatile int *abort_flag = reinterpret_cast<volatile int *>(misc + 1);
+    uint32_t *nx_bits = reinterpret_cast<uint32_t *>(misc + 4);
+
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int rank = n_split > 1 ? (int)cluster_rank() : 0;
+    const int mt = blockIdx.x / n_split;
+    const int nk = p.d_in / kGBK;
+    const int kb0 = (int)((int64_t)nk * rank / n_split);
+    const int kbn = (int)((int64_t)nk * (rank + 1) / n_split) - kb0;
+
+    if (tid == 0) {
+        for (int s = 0; s < C::kStages; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        mbar_init(acc_full, 1);
+        *abort_flag = 0;
+        fence_mbar_init();
+    }
+    if (warp == 1) {
+        tmem_alloc(reinterpret_cast<uint32_t *>(&misc[0]), C::kTmemCols);
+        tmem_relinquish();
+    }
+    pdl_wait();
+    pdl_trigger();
+    if (warp == 2) {
+        uint32_t kinds = 0;  // bit 0: ordinary rows, bit 1: Nexus rows
+        for (int w = 0; w < (NT + 31) / 32; ++w) {
+            const int t = w * 32 + lane;
+            const bool in = t < p.T;
+            const bool nx = in && role[t] == SONIC_ROLE_NEXUS;
+            const uint32_t b = __ballot_sync(0xffffffffu, nx);
+            if (__any_sync(0xffffffffu, in && !nx)) kinds |= 1;
+            if (b) kinds |= 2;
+            if (lane == 0) nx_bits[w] = b;
+        }
+        if (lane == 0) misc[2] = (int32_t)kinds;
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = static_cast<uint32_t>(misc[0]);
+    const int kinds = timed_out(p.status) ? 0 : misc[2];
+    const int n_it = (kinds == 3 ? 2 : kinds ? 1 : 0) * kbn;  // stages of the whole call
+
+    int issued = 0;
+    if (warp == 0) {
+        if (lane == 0) {
+            tma_prefetch_desc(&tmX);
+            for (int it = 0; it < n_it; ++it) {
+                const int s = it % C::kStages;
+                if (it >= C::kStages &&
+                    !mbar_wait(&empty[s], ((it / C::kStages) - 1) & 1, p.status, abort_flag))
+                    break;
+                const bool second = it >= kbn;
+                const CUtensorMap *tw = (second || kinds == 2) ? &tmWn : &tmW;
+                const int k = (kb0 + (second ? it - kbn : it)) * kGBK;
+                uint8_t *w = smem + s * C::kStageBytes;
+                mbar_arrive_expect_tx(&full[s], C::kStageBytes);
+                tma_load_4d(w, tw, &full[s], k, mt * kHalfN, 0, 0);
+                tma_load_4d(w + C::kWBytes, &tmX, &full[s], k, 0, 0, 0);
+                issued = it + 1;
+            }
+        }
+    } else if (warp == 1) {
+        if (lane == 0) {
+            constexpr uint32_t idesc = idesc_bf16_f32(kHalfN, NT, 0, 0);
+            const uint32_t base = smem_u32(smem);
+            for (int it = 0; it < n_it; ++it) {
+                const int s = it % C::kStages;
+                if (!mbar_wait(&full[s], (it / C::kStages) & 1, p.status, abort_flag)) break;
+                tc_fence_after();
+                const uint32_t w_addr = base + s * C::kStageBytes, x_addr = w_addr + C::kWBytes;
+                const uint32_t acc = tmem + (it >= kbn ? NT : 0);
+                const bool start = it == 0 || it == kbn;
+#pragma unroll
+                for (int kk = 0; kk < kGBK / 16; ++kk)
+                    tc_mma_ss(acc, smem_desc_sw128(w_addr + kk * 32, 16, 1024),
+                              smem_desc_sw128(x_addr + kk * 32, 16, 1024), idesc,
+                              (!start || kk > 0) ? 1u : 0u);
+                tc_commit(&empty[s]);
+            }
+            // arrives once every MMA issued has finished (after an abort too:
+            // tensor memory is freed after it)
+            tc_commit(acc_full);
+            mbar_drain(acc_full, 0);
+        }
+    }
+    tc_fence_before();
+    __syncthreads();  // every MMA is done and every copy has been read: the ring is free
+    tc_fence_after();
+    if (*abort_flag) {  // (block-uniform by now) the copies in flight land first
+        if (warp == 0 && lane == 0)
+            for (int u = max(0, issued - C::kStages); u < issued; ++u)
+                mbar_drain(&full[u % C::kStages], (u / C::kStages) & 1);
+        __syncthreads();
+    }
+
+    // partial sums [row][128 weight rows] over the ring (thread = weight row =
+    // TMEM lane), each row of X taking the accumulator of its kind
+    float *part = reinterpret_cast<float *>(smem);
+    if (warp >= 2 && n_it > 0) {
+        const int quarter = warp & 3, r = quarter * 32 + lane;
+        const uint32_t lane_base = static_cast<uint32_t>(quarter * 32) << 16;
+#pragma unroll 1
+        for (int c = 0; c < NT / 16 && c * 16 < p.T; ++c) {
+            uint32_t v[16];
+            tmem_ld16(tmem + lane_base + c * 16, v);
+            if (kinds == 3) {
+                uint32_t u[16];
+                tmem_ld16(tmem + lane_base + NT + c * 16, u);
+                tmem_ld_wait();
+                reg_fence16(u);
+                reg_fence16(v);
+                const uint32_t bits = nx_bits[c >> 1] >> ((c & 1) * 16);
+#pragma unroll
+                for (int x = 0; x < 16; ++x)
+                    if ((bits >> x) & 1) v[x] = u[x];
+            }
+            tmem_ld_wait();
+            reg_fence16(v);
+#pragma unroll
+            for (int x = 0; x < 16; ++x)
+                part[(c * 16 + x) * kHalfN + r] = __uint_as_float(v[x]);
+        }
+    }
+    tc_fence_before();
+    if (n_split > 1) cluster_sync_all();
+    __syncthreads();
+    tc_fence_after();
+    if (warp == 1) tmem_dealloc(tmem, C::kTmemCols);
+    // rank q adds and writes rows q, q + S, ... : 8 columns per thread
+    if (n_it > 0) {
+        const int n_rows = (p.T - rank + n_split - 1) / n_split;
+        for (int i = tid; i < n_rows * (kHalfN / 8); i += kGThreads) {
+            const int t = rank + n_split * (i / (kHalfN / 8)), c = (i % (kHalfN / 8)) * 8;
+            const int col = mt * kHalfN + c;
+            if (col >= p.d_out) continue;
+            const float *mine = part + t * kHalfN + c;
+            float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
+            for (int q = 0; q < n_split; ++q) {
+                const uint32_t at = n_split > 1 ? smem_in_rank(mine, q) : smem_u32(mine);
+                const float4 x = ld_cluster_f4(at), y = ld_cluster_f4(at + 16);
+                a.x += x.x; a.y += x.y; a.z += x.z; a.w += x.w;
+                b.x += y.x; b.y += y.y; b.z += y.z; b.w += y.w;
+            }
+            int k = 0;
+#pragma unroll
+            for (int q = 1; q < kMaxParts; ++q)
+                if (q < p.n_parts && col >= p.part[q].col0) k = q;
+            const GemmPart &pt = p.part[k];
+            const int64_t row = pt.scatter ? p.dst_row[t] : t;
+            if (row < 0 || row >= pt.rows) {  // outside the part: not written
+                set_status(p.status, SONIC_ERR_CAPACITY);
+                continue;
+            }
+            *reinterpret_cast<uint4 *>(pt.base + row * pt.stride + (col - pt.col0)) =
+                make_uint4(pack_bf16x2(a.x, a.y), pack_bf16x2(a.z, a.w), pack_bf16x2(b.x, b.y),
+                           pack_bf16x2(b.z, b.w));
+        }
+    }
+    if (n_split > 1) cluster_sync_all();  // no CTA leaves while another reads its sums
+}
+
+// CTAs per 128 weight rows: the largest cluster with which all `tiles` clusters are
+// resident at once (one CTA per SM; clusters don't span the GPU's SM groups, so
+// fewer fit than SMs / size), at most 8 and at most one per four reduction steps.
+template <int NT>
+int small_split(int tiles, int nk) {
+    // clusters of each size that fit, per device (0: not asked yet)
+    static std::atomic<int> most[64][9];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 1;
+    for (int s = 8; s > 1; --s) {
+        if (s * 4 > nk) continue;
+        int fit = dev < 64 ? most[dev][s].load(std::memory_order_relaxed) : 0;
+        if (fit == 0) {
+            cudaLaunchAttribute at{};
+            at.id = cudaLaunchAttributeClusterDimension;
+            at.val.clusterDim.x = s;
+            at.val.clusterDim.y = at.val.clusterDim.z = 1;
+            cudaLaunchConfig_t cfg{};
+            cfg.gridDim = dim3(s);
+            cfg.blockDim = dim3(kGThreads);
+            cfg.dynamicSmemBytes = SmallCfg<NT>::kSmem;
+            cfg.attrs = &at;
+            cfg.numAttrs = 1;
+            if (cudaOccupancyMaxActiveClusters(&fit, routed_small_kernel<NT>, &cfg) != cudaSuccess) {
+                (void)cudaGetLastError();
+                fit = 0;
+            }
+            if (dev < 64) most[dev][s].store(fit > 0 ? fit : -1, std::memory_order_relaxed);
+        }
+        if (fit >= tiles) return s;
+    }
+    return 1;
+}
+
+template <int NT>
+cudaError_t launch_small(const uint16_t *X, const CUtensorMap &tW, const CUtensorMap &tWn,
+                         const uint8_t *role, const GemmParams &p, int64_t x_row_stride,
+                         cudaStream_t stream) {
+    const uint64_t dims[4] = {(uint64_t)p.d_in, (uint64_t)p.T, 1, 1};
+    const uint64_t str[3] = {(uint64_t)x_row_stride * 2, (uint64_t)x_row_stride * 2 * p.T,
+                             (uint64_t)x_row_stride * 2 * p.T};
+    const uint32_t box[4] = {kGBK, NT, 1, 1};
+    CUtensorMap tX;
+    if (!make_tmap_bf16_4d(&tX, X, dims, str, box)) return cudaErrorInvalidValue;
+    constexpr size_t smem = SmallCfg<NT>::kSmem;
+    static_assert(smem <= 232448, "routed GEMM shared memory");
+    cudaError_t e = cudaFuncSetAttribute(routed_small_kernel<NT>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    const int tiles = (p.d_out + kHalfN - 1) / kHalfN;
+    const int split = small_split<NT>(tiles, p.d_in / kGBK);
+    return launch_pdl(routed_small_kernel<NT>, dim3(tiles * split), kGThreads, smem, stream, split,
+                      tX, tW, tWn, role, p, split);
+}
+
 struct RlWorkspace {
     size_t counts, groups, perm, xg, total;
 };
@@ -565,11 +824,31 @@ extern "C" sonic_status_t sonic_routed_linear(const uint16_t *X, const uint16_t 
     const uint64_t xdims[4] = {(uint64_t)a->d_in, (uint64_t)T, 1, 1};
     const uint64_t xstr[3] = {(uint64_t)a->x_row_stride * 2, (uint64_t)a->x_row_stride * 2 * T,
                               (uint64_t)a->x_row_stride * 2 * T};
+    p.groups = groups;
+    p.perm = perm;
+    p.dst_row = a->dst_row;
+    p.n_parts = a->n_parts;
+    p.T = T;
+    p.d_in = a->d_in;
+    p.d_out = a->d_out;
+    p.n_tiles_n = (a->d_out + kGBN - 1) / kGBN;
+    p.status = a->status;
     CUtensorMap tA, tX, tW, tWn;
-    if (!make_tmap_bf16_4d(&tA, Xg, adims, astr, abox) ||
-        !make_tmap_bf16_4d(&tX, X, xdims, xstr, abox) ||
-        !make_tmap_bf16_4d(&tW, W, wdims, wstr, wbox) ||
+    if (!make_tmap_bf16_4d(&tW, W, wdims, wstr, wbox) ||
         !make_tmap_bf16_4d(&tWn, W_nexus, wdims, wstr, wbox))
+        return SONIC_ERR_INVALID_ARGUMENT;
+    if (T <= kSmallRows) {
+        const cudaError_t e = T <= 16    ? launch_small<16>(X, tW, tWn, role, p, a->x_row_stride, stream)
+                              : T <= 32  ? launch_small<32>(X, tW, tWn, role, p, a->x_row_stride, stream)
+                              : T <= 64  ? launch_small<64>(X, tW, tWn, role, p, a->x_row_stride, stream)
+                              : T <= 128 ? launch_small<128>(X, tW, tWn, role, p, a->x_row_stride, stream)
+                                         : launch_small<192>(X, tW, tWn, role, p, a->x_row_stride, stream);
+        return e == cudaSuccess             ? SONIC_OK
+               : e == cudaErrorInvalidValue ? SONIC_ERR_INVALID_ARGUMENT
+                                            : SONIC_ERR_CUDA;
+    }
+    if (!make_tmap_bf16_4d(&tA, Xg, adims, astr, abox) ||
+        !make_tmap_bf16_4d(&tX, X, xdims, xstr, abox))
         return SONIC_ERR_INVALID_ARGUMENT;
 
     role_count_kernel<<<chunks, 256, 0, stream>>>(role, T, counts);
@@ -581,15 +860,6 @@ extern "C" sonic_status_t sonic_routed_linear(const uint16_t *X, const uint16_t 
         reinterpret_cast<const uint8_t *>(X), a->x_row_stride * 2, T, (int64_t)a->d_in * 2, perm,
         groups, reinterpret_cast<uint8_t *>(Xg));
 
-    p.groups = groups;
-    p.perm = perm;
-    p.dst_row = a->dst_row;
-    p.n_parts = a->n_parts;
-    p.T = T;
-    p.d_in = a->d_in;
-    p.d_out = a->d_out;
-    p.n_tiles_n = (a->d_out + kGBN - 1) / kGBN;
-    p.status = a->status;
     const long long max_tiles = ((long long)(T + kGBM - 1) / kGBM + 1) * p.n_tiles_n;
     const int pairs = (int)(max_tiles < sms / 2 ? max_tiles : sms / 2);
     const int blocks = 2 * (pairs > 0 ? pairs : 1);
