@@ -14,6 +14,8 @@
 //                  accumulator) goes to the workspace.  head_dim 64 and 128.
 //   decode_combine log-sum-exp merge of the chunks of each (layer, seq, head).
 // K and V are read exactly once from HBM; softmax runs in base 2.
+#include <type_traits>
+
 #include "sonic_dev.cuh"
 #include "sonic_host.h"
 
@@ -40,9 +42,69 @@ struct DecParams {
     int B, Hq, Hkv, G;
     int64_t total_kv_rows;  // rows of K_ret, V_ret (and role) per layer
     int64_t q_ls, o_ls;
-    int chunk_len, max_chunks;
+    int n_layers;
+    int chunk_len, max_chunks;  // split by chunks; a sequence is clipped at their product
+    int groups;                 // > 0: split into equal shares (see Share), this many per KV head
+    int slot_heads;             // query heads of a unit
+    int slot_stride;            // partial slots from one of them to the next
     float scale_log2;
 };
+
+// Rows of sequence b: clipped to the plan's limit; none when they fall outside
+// the cache (such a sequence is refused, nothing of it is read).
+__device__ __forceinline__ int seq_keys(const DecParams &p, int raw_len, int start) {
+    const int len = min(max(raw_len, 0), p.max_chunks * p.chunk_len);
+    return (start < 0 || (int64_t)start + len > p.total_kv_rows) ? 0 : len;
+}
+__device__ __forceinline__ bool seq_refused(const DecParams &p, int raw_len, int start) {
+    return start < 0 ||
+           (int64_t)start + min(max(raw_len, 0), p.max_chunks * p.chunk_len) > p.total_kv_rows;
+}
+
+// Equal shares.  The keys of all (layer, sequence) pairs form one line of n
+// keys (layer-major, the sequences' lengths one after another); group g of the
+// `groups` blocks of a KV head takes keys [bound(g), bound(g + 1)).  Cuts lie
+// `per` keys apart, moved to a sequence's end where that is less than kSnap keys
+// away, so no piece is shorter than that unless its sequence is.
+constexpr int kMinShare = 64;
+constexpr int kSnap = 32;
+
+__device__ __forceinline__ int share_of(int n, int groups) {
+    const int per = ((n + groups - 1) / groups + 15) & ~15;
+    return per < kMinShare ? kMinShare : per;
+}
+
+// A cut at offset `off` of a sequence of `len` keys, moved (off < len).
+__device__ __forceinline__ int snap(int off, int len) {
+    return off < kSnap ? 0 : (len - off < kSnap ? len : off);
+}
+
+// The sequence holding key x of one layer's line (x < the lengths' sum), found by
+// a whole warp, and x's offset in it; len(b) gives the length of sequence b.
+template <typename F>
+__device__ __forceinline__ void find_seq(int B, F len, int x, int &seq, int &off) {
+    const int lane = threadIdx.x & 31;
+    int base = 0;
+    for (int b0 = 0; b0 < B; b0 += 32) {
+        const int v = b0 + lane < B ? len(b0 + lane) : 0;
+        int incl = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += u;
+        }
+        const unsigned past = __ballot_sync(0xffffffffu, base + incl > x);
+        if (past) {
+            const int at = __ffs(past) - 1;
+            seq = b0 + at;
+            off = x - base - __shfl_sync(0xffffffffu, incl - v, at);
+            return;
+        }
+        base += __shfl_sync(0xffffffffu, incl, 31);
+    }
+    seq = B;
+    off = 0;
+}
 
 // Maximum of v over the 32 lanes of the warp, in one instruction.
 __device__ __forceinline__ float warp_max(float v) {
@@ -91,64 +153,57 @@ struct TcCfg {
     static constexpr int kOffN = kOffL + 4 * kTcN * 4;           // [4][16] float
     static constexpr int kOffBar = kOffN + 4 * kTcN * 4;
     static constexpr int kNumBars = 2 * kTcStages + 24;  // the pointers carved out below
-    static constexpr int kOffMisc = kOffBar + kNumBars * 8;
+    static constexpr int kOffMisc = kOffBar + (kNumBars * 8 + 15) / 16 * 16;
     static constexpr int kSeqCache = 1024;                       // sequences whose lens/kv_start
-    static constexpr int kOffSeq = kOffMisc + 128;               // are cached: [2][1024] int32
+    static constexpr int kOffSeq = kOffMisc + 16 + 32 * 4;       // are cached: [2][1024] int32
     static constexpr size_t kSmem = 1024 + kOffSeq + 2 * kSeqCache * 4;
 };
 constexpr int kUnitSlots = 4;  // claimed-unit queue between the producer and the others
 
-// Unit u: (key chunk, KV head, sequence, layer), KV head fastest.  A unit whose
-// chunk starts past the sequence's end has no keys.
+// A unit of work: some keys of one (layer, sequence, KV head).
 struct TcUnit {
-    int u, kvh, chunk, b, layer, nkeys, ntiles, row0, len;
+    int nkeys, row0, b, layer, kvh;
+    int ntiles;
+    // its first query head's slot of the partials; -1: the unit holds all keys of its
+    // sequence, O is written directly
+    int64_t slot;
 };
 
-// The indices of unit w.u and its tile count (from w.nkeys).
-__device__ __forceinline__ void tc_coords(const DecParams &p, int units_x, TcUnit &w) {
-    const int x = w.u % units_x, y = w.u / units_x;
-    w.kvh = x % p.Hkv;
-    w.chunk = x / p.Hkv;
-    w.b = y % p.B;
-    w.layer = y / p.B;
-    w.ntiles = (w.nkeys + kTcKeys - 1) / kTcKeys;
-}
-
+// Unit u of the split by chunks: (key chunk, KV head, sequence, layer), KV head
+// fastest.  False when the chunk starts past the sequence's end.
 // seq_len / seq_start: the sequences' lengths and first rows cached in shared
 // memory (B <= kSeqCache), or NULL to read them from global memory.
-__device__ __forceinline__ bool tc_unit(const DecParams &p, int units_x, int u, TcUnit &w,
+__device__ __forceinline__ bool tc_unit(const DecParams &p, int units_x, int u, int n_heads, TcUnit &w,
                                         const int32_t *seq_len, const int32_t *seq_start) {
     const int x = u % units_x, y = u / units_x;
-    w.u = u;
     w.kvh = x % p.Hkv;
-    w.chunk = x / p.Hkv;
+    const int chunk = x / p.Hkv;
     w.b = y % p.B;
     w.layer = y / p.B;
-    int len = seq_len != nullptr ? seq_len[w.b] : p.lens[w.b];
-    len = min(max(len, 0), p.max_chunks * p.chunk_len);
+    const int raw = seq_len != nullptr ? seq_len[w.b] : p.lens[w.b];
     const int start = seq_start != nullptr ? seq_start[w.b] : p.kv_start[w.b];
-    if (start < 0 || (int64_t)start + len > p.total_kv_rows) {
-        // rows outside the cache: the sequence is refused, nothing is read
-        if (w.chunk == 0 && w.kvh == 0) set_status(p.status, SONIC_ERR_INVALID_ARGUMENT);
-        len = 0;
-    }
-    const int key0 = w.chunk * p.chunk_len;
-    w.len = len;
+    const int len = seq_keys(p, raw, start);
+    if (chunk == 0 && w.kvh == 0 && seq_refused(p, raw, start))
+        set_status(p.status, SONIC_ERR_INVALID_ARGUMENT);
+    const int key0 = chunk * p.chunk_len;
     w.nkeys = max(min(p.chunk_len, len - key0), 0);
-    w.ntiles = (w.nkeys + kTcKeys - 1) / kTcKeys;
     w.row0 = start + key0;
+    w.slot = len <= p.chunk_len
+                 ? -1
+                 : (((int64_t)w.layer * p.B + w.b) * p.Hq + w.kvh * n_heads) * p.max_chunks + chunk;
     return w.nkeys > 0;
 }
 
 // D = 64 or 128.  The stage layout is the D = 128 one.  At D = 64 either the
-// second 64-column half of each K and V tile is never loaded and stays zero
-// (the ring is zeroed at kernel start), or (kPair, when G <= 8) a unit takes
+// second 64-column half of each K and V tile is never loaded (whatever it holds
+// reaches rows 64-127 of O^T alone, which are never read), or (kPair, when G <= 8) a unit takes
 // two KV heads: head 2i's rows fill the first half and head 2i+1's the second,
 // the 16 staged query heads hold both heads' G queries, and S^T and O^T get a
 // region per KV head (query column v belongs to head 2i for v < G, to head
 // 2i+1 after), so a 128-key tile carries as many bytes as at D = 128 for the
-// same per-tile softmax work.  O^T += V^T P^T keeps M = 128 either way (rows
-// 64-127 accumulate zeros, or the other half's data; they are never written).
+// same per-tile softmax work.  O^T += V^T P^T keeps M = 128 either way.  The P
+// columns of heads past the unit's are not written either: they reach their own
+// columns of O^T alone.
 template <int D, int GT, bool kPair>
 __global__ void __launch_bounds__(kTcThreads, 1)
 decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
@@ -186,36 +241,14 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     uint64_t *uq_full = o_free + 2;    // [kUnitSlots] a claimed unit is in its slot
     uint64_t *uq_empty = uq_full + kUnitSlots;  // [kUnitSlots] the issuer and 4 warps read it
     int32_t *misc = reinterpret_cast<int32_t *>(smem + C::kOffMisc);
-    // [kUnitSlots][4]: unit index (-1: no more), its keys, first key row, sequence length
-    volatile int32_t *unit_q = misc + 4;
+    // [kUnitSlots][2]: (keys (0: no more units), first key row, sequence, layer), (KV head,
+    // low and high word of the slot)
+    int4 *unit_q = reinterpret_cast<int4 *>(misc + 4);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(misc + 1);
 
     const int G = p.G;
+    const int Gv = kPair ? 2 * G : G;  // query columns of a unit
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    if (timed_out(p.status)) return;
-    if (tid == 0) {
-        // a sequence longer than the plan allows is clipped, and reported
-        for (int b = blockIdx.x; b < p.B; b += gridDim.x)
-            if (p.lens[b] > p.max_chunks * p.chunk_len) set_status(p.status, SONIC_ERR_INVALID_ARGUMENT);
-    }
-
-    // The P buffers zeroed (rows >= GT stay zero), and the K/V ring: rows a
-    // partial tile does not load keep older, finite data, which P = 0 cancels.
-    for (int i = tid; i < 2 * C::kPBytes / 16; i += blockDim.x)
-        reinterpret_cast<uint4 *>(P_s)[i] = make_uint4(0, 0, 0, 0);
-    for (int i = tid; i < kTcStages * C::kStageBytes / 16; i += blockDim.x)
-        reinterpret_cast<uint4 *>(smem)[i] = make_uint4(0, 0, 0, 0);
-    // the sequences' lengths and first rows, for claiming units without
-    // global loads on the producer's path
-    int32_t *seq_len = nullptr, *seq_start = nullptr;
-    if (p.B <= C::kSeqCache) {
-        seq_len = reinterpret_cast<int32_t *>(smem + C::kOffSeq);
-        seq_start = seq_len + C::kSeqCache;
-        for (int b = tid; b < p.B; b += blockDim.x) {
-            seq_len[b] = p.lens[b];
-            seq_start[b] = p.kv_start[b];
-        }
-    }
     if (tid == 0) {
         for (int s = 0; s < kTcStages; ++s) {
             mbar_init(&full[s], 1);
@@ -242,72 +275,148 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
         *abort_flag = 0;
         fence_mbar_init();
     }
+    if (tid == 0) {
+        tma_prefetch_desc(&tmK);
+        tma_prefetch_desc(&tmV);
+        tma_prefetch_desc(&tmK16);
+        tma_prefetch_desc(&tmV16);
+        tma_prefetch_desc(&tmQ);
+    }
     if (warp == 1) {
         tmem_alloc(reinterpret_cast<uint32_t *>(&misc[0]), kTmemCols);
         tmem_relinquish();
     }
-    fence_proxy_async_smem();
+    pdl_wait();
+    pdl_trigger();
+    // the sequences' lengths and first rows, for the producer to find its units
+    // without global loads on its path; a sequence longer than the plan allows is
+    // clipped, and reported
+    int32_t *seq_len = nullptr, *seq_start = nullptr;
+    if (p.B <= C::kSeqCache) {
+        seq_len = reinterpret_cast<int32_t *>(smem + C::kOffSeq);
+        seq_start = seq_len + C::kSeqCache;
+        for (int b = tid; b < p.B; b += blockDim.x) {
+            const int raw = p.lens[b], start = p.kv_start[b];
+            if (blockIdx.x == 0 && raw > p.max_chunks * p.chunk_len)
+                set_status(p.status, SONIC_ERR_INVALID_ARGUMENT);
+            seq_len[b] = raw;
+            seq_start[b] = start;
+            if (p.groups > 0) {
+                seq_len[b] = seq_keys(p, raw, start);
+                if (blockIdx.x == 0 && seq_refused(p, raw, start))
+                    set_status(p.status, SONIC_ERR_INVALID_ARGUMENT);
+            }
+        }
+    } else if (tid == 0) {
+        for (int b = blockIdx.x; b < p.B; b += gridDim.x)
+            if (p.lens[b] > p.max_chunks * p.chunk_len) set_status(p.status, SONIC_ERR_INVALID_ARGUMENT);
+    }
+    if (tid == 32) misc[2] = timed_out(p.status);  // no units for this block
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    const bool dead = misc[2] != 0;
     const uint32_t tmem = static_cast<uint32_t>(misc[0]);
     // TMEM: S^T [2] then O^T [2], kSStride columns each (a 16-column region
     // per KV head of the unit)
     const uint32_t tS = tmem, tO = tmem + 2 * kSStride;
-    const int Gv = kPair ? 2 * G : G;  // query columns of a unit
-    // The k-th claimed unit (w.u = -1: none left, or a wait gave up), from
-    // shared memory: the consumers never touch global memory for it.  Each
-    // reader (the issuer, lane 0 of each softmax warp) frees the slot.
+    // The k-th claimed unit (false: none left, or a wait gave up), from shared
+    // memory: the consumers never touch global memory for it.  Called by one
+    // thread (the issuer) or a whole warp (softmax); the caller frees the slot.
     auto read_unit = [&](int k, TcUnit &w) -> bool {
         const int slot = k & (kUnitSlots - 1);
-        w.u = -1;
         if (!mbar_wait(&uq_full[slot], (k / kUnitSlots) & 1, p.status, abort_flag)) return false;
-        const volatile int32_t *q = unit_q + slot * 4;
-        w.u = q[0];
-        w.nkeys = q[1];
-        w.row0 = q[2];
-        w.len = q[3];
-        mbar_arrive(&uq_empty[slot]);
-        return w.u >= 0;
+        const int4 a = unit_q[slot * 2], c = unit_q[slot * 2 + 1];
+        w.nkeys = a.x;
+        w.row0 = a.y;
+        w.b = a.z;
+        w.layer = a.w;
+        w.kvh = c.x;
+        w.slot = ((int64_t)c.z << 32) | (uint32_t)c.y;
+        w.ntiles = (w.nkeys + kTcKeys - 1) / kTcKeys;
+        return w.nkeys > 0;
     };
 
     int issued_q = 0, issued_kv = 0;  // copies the producer issued (for the drain)
     if (warp == 0) {
         // ------------------------------------------------------------ producer
-        if (lane == 0) {
-            tma_prefetch_desc(&tmK);
-            tma_prefetch_desc(&tmV);
+        // Equal shares: this block's keys [cur, end) of the line, cur at offset off of
+        // sequence sb, layer sl.
+        int cur = 0, end = 0, off = 0, sb = 0, sl = 0;
+        if (p.groups > 0 && !dead) {
+            auto len_of = [&](int b) { return seq_len[b]; };
+            int sum = 0;
+            for (int b = lane; b < p.B; b += 32) sum += seq_len[b];
+            sum = __reduce_add_sync(0xffffffffu, sum);
+            const int n = sum * p.n_layers, per = share_of(n, p.groups);
+            auto cut = [&](int g, int &layer, int &b, int &o) -> int {
+                const long long x = (long long)g * per;
+                if (x >= n) return n;
+                layer = (int)x / sum;
+                find_seq(p.B, len_of, (int)x - layer * sum, b, o);
+                const int to = snap(o, seq_len[b]), at = (int)x - o + to;
+                o = to;
+                return at;
+            };
+            const int grp = (int)blockIdx.x / p.Hkv;
+            int l1, b1, o1;
+            cur = cut(grp, sl, sb, off);
+            end = cut(grp + 1, l1, b1, o1);
         }
-        // Lane 0 claims units from the counter, publishes each in the unit
+        // Lane 0 finds its units (equal shares) or claims them from the counter, publishes each in the unit
         // queue and streams its q (one TMA box of 16 heads: rows past the
         // group's G heads are other heads' q or zeros, whose S^T columns the
         // softmax never reads) and its K/V tiles.  The claim of unit k + 1 is
         // sent before unit k's copies are queued; its answer is needed only
         // after them.
         if (lane == 0) {
-            tma_prefetch_desc(&tmQ);
             int T = 0;  // K/V tiles issued
-            int pending = atomicAdd(unit_counter, 1);
+            auto next_share = [&](TcUnit &w) -> bool {
+                while (cur < end) {
+                    const int len = seq_len[sb], take = min(len - off, end - cur);
+                    w.b = sb;
+                    w.layer = sl;
+                    w.kvh = (int)blockIdx.x % p.Hkv;
+                    w.nkeys = take;
+                    w.row0 = seq_start[sb] + off;
+                    // a block cuts at most two sequences: the first (from the middle
+                    // on) has slot 0, the last (from its start) slot 1
+                    w.slot = take == len ? -1 : ((int64_t)blockIdx.x * 2 + (off > 0 ? 0 : 1)) * Gv;
+                    cur += take;  // (take is 0 where the cut was moved to the sequence's end)
+                    off = 0;
+                    if (++sb == p.B) {
+                        sb = 0;
+                        ++sl;
+                    }
+                    if (take > 0) return true;
+                }
+                return false;
+            };
+            int pending = p.groups > 0 || dead ? n_units : atomicAdd(unit_counter, 1);
             for (int k = 0;; ++k) {
                 const int slot = k & (kUnitSlots - 1);
                 bool ok = k < kUnitSlots ||
                           mbar_wait(&uq_empty[slot], ((k / kUnitSlots) - 1) & 1, p.status, abort_flag);
-                int u = -1;
+                bool have = false;
                 TcUnit w;
+                w.nkeys = 0;
                 if (ok) {
-                    u = pending;
-                    while (u < n_units && !tc_unit(p, units_x, u, w, seq_len, seq_start))
-                        u = atomicAdd(unit_counter, 1);
-                    if (u >= n_units) u = -1;
+                    if (p.groups > 0) {
+                        have = next_share(w);
+                    } else {
+                        int u = pending;
+                        while (u < n_units && !tc_unit(p, units_x, u, Gv, w, seq_len, seq_start))
+                            u = atomicAdd(unit_counter, 1);
+                        have = u < n_units;
+                    }
                 }
-                volatile int32_t *q = unit_q + slot * 4;
-                q[0] = u;
-                q[1] = w.nkeys;
-                q[2] = w.row0;
-                q[3] = w.len;
+                unit_q[slot * 2] = make_int4(have ? w.nkeys : 0, w.row0, w.b, w.layer);
+                unit_q[slot * 2 + 1] =
+                    make_int4(w.kvh, (int)(uint32_t)w.slot, (int)(w.slot >> 32), 0);
                 mbar_arrive(&uq_full[slot]);  // release: the slot is written
-                if (u < 0) break;
-                pending = atomicAdd(unit_counter, 1);
+                if (!have) break;
+                w.ntiles = (w.nkeys + kTcKeys - 1) / kTcKeys;
+                if (p.groups == 0) pending = atomicAdd(unit_counter, 1);
                 // q into buffer k & 1 once the S^T MMAs of unit k - 2 no longer read it
                 const int qb = k & 1;
                 if (k >= 2 && !mbar_wait(&q_empty[qb], ((k >> 1) - 1) & 1, p.status, abort_flag))
@@ -405,11 +514,13 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
             };
             TcUnit w, nx;
             int T = 0, k = 0;
-            bool ok = read_unit(0, w);
-            if (ok) {
-                tc_coords(p, units_x, w);
-                ok = issue_s(0, 0, 0, w.ntiles);
-            }
+            auto take_unit = [&](int k, TcUnit &u) -> bool {
+                const bool have = read_unit(k, u);
+                mbar_arrive(&uq_empty[k & (kUnitSlots - 1)]);
+                return have;
+            };
+            bool ok = take_unit(0, w);
+            if (ok) ok = issue_s(0, 0, 0, w.ntiles);
             for (bool more = true; ok && more; ++k) {
                 bool has_next = false;
                 for (int t = 0; ok && t < w.ntiles; ++t, ++T) {
@@ -421,9 +532,8 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                     int nk = k, nt1 = t + 1, nnt = w.ntiles;
                     bool next_tile = t + 1 < w.ntiles;
                     if (!next_tile) {
-                        has_next = read_unit(k + 1, nx);
+                        has_next = take_unit(k + 1, nx);
                         if (has_next) {
-                            tc_coords(p, units_x, nx);
                             next_tile = true;
                             nk = k + 1;
                             nt1 = 0;
@@ -525,7 +635,6 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
             // O^T of this unit is in registers and lred read: the buffers are free
             tc_fence_before();
             mbar_arrive(&o_free[k & 1]);
-            const int n_chunks = (w.len + p.chunk_len - 1) / p.chunk_len;
             const int hb = (kPair ? 2 * w.kvh : w.kvh) * G;  // the unit's first query head
             const int64_t unit0 = ((int64_t)w.layer * p.B + w.b) * p.Hq + hb;
 #pragma unroll
@@ -533,14 +642,14 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                 if (g >= Gv) break;
                 const float L = Lg[g];
                 const float a = __uint_as_float(o[g]);
-                if (n_chunks == 1) {
+                if (w.slot < 0) {
                     uint16_t *op =
                         p.O + w.layer * p.o_ls + ((int64_t)w.b * p.Hq + hb + g) * D;
                     if (r < D) op[r] = __bfloat16_as_ushort(__float2bfloat16_rn(a / L));
                     if (r == 0 && p.lse != nullptr) p.lse[unit0 + g] = (m[g] + __log2f(L)) * kLn2;
                     if (r == 0 && want_nx) p.nexus_mass[unit0 + g] = Ng[g] / L;
                 } else {
-                    const int64_t slot = (unit0 + g) * p.max_chunks + w.chunk;
+                    const int64_t slot = w.slot + (int64_t)g * p.slot_stride;
                     if (r < D) p.part_acc[slot * D + r] = a;
                     if (r == 0) {
                         p.part_ml[slot * 2 + 0] = m[g];
@@ -557,13 +666,11 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
         float mp[GT], lp[GT], np[GT];
         for (int k = 0; ok; ++k) {
             TcUnit w;
-            if (lane == 0) read_unit(k, w);
-            w.u = __shfl_sync(0xffffffffu, w.u, 0);
-            if (w.u < 0) break;
-            w.nkeys = __shfl_sync(0xffffffffu, w.nkeys, 0);
-            w.row0 = __shfl_sync(0xffffffffu, w.row0, 0);
-            w.len = __shfl_sync(0xffffffffu, w.len, 0);
-            tc_coords(p, units_x, w);
+            const bool have = read_unit(k, w);
+            // every lane has read the slot before lane 0 frees it (and none goes on
+            // where another's wait gave up)
+            if (!__all_sync(0xffffffffu, have)) break;
+            if (lane == 0) mbar_arrive(&uq_empty[k & (kUnitSlots - 1)]);
             const uint32_t tOk = tO + (k & 1) * kSStride;
             float m[GT], l[GT], n[GT];
 #pragma unroll
@@ -637,10 +744,10 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                     if (want_nx) n[g] = n[g] * alpha[g] + (isn ? __bfloat162float(pr) : 0.f);
                     *reinterpret_cast<__nv_bfloat16 *>(pb + g * 128 + ((jj ^ (g & 7)) << 4)) = pr;
                 }
-                if (!valid && r < ((w.nkeys - t * kTcKeys + 15) & ~15)) {
-                    // rows a partial tile loaded past the unit's keys (another
-                    // sequence's, or junk): zero their V, so 0 * garbage cannot
-                    // reach O
+                if (!valid) {
+                    // rows of a partial tile past the unit's keys (another sequence's,
+                    // junk, or what shared memory held): zero their V, so 0 * garbage
+                    // cannot reach O (their K only makes scores that are masked)
                     uint8_t *vrow =
                         smem + (T % kTcStages) * C::kStageBytes + C::kTileBytes + r * 128;
 #pragma unroll
@@ -707,10 +814,14 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     if (warp == 1) tmem_dealloc(tmem, kTmemCols);
 }
 
-// One warp per (layer, sequence, query head).
+// One warp per (layer, sequence, query head): the log-sum-exp merge of its pieces
+// (chunks, or the shares its sequence is cut into).  A warp's lanes fetch the pieces'
+// maxima and sums side by side, then every accumulator load is independent of them.
 template <int D>
 __global__ void __launch_bounds__(128)
 decode_combine_kernel(const DecParams p, int n_layers) {
+    pdl_wait();
+    pdl_trigger();
     const int64_t unit = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     const int64_t n_units = (int64_t)n_layers * p.B * p.Hq;
@@ -718,38 +829,93 @@ decode_combine_kernel(const DecParams p, int n_layers) {
     const int h = (int)(unit % p.Hq);
     const int64_t lb = unit / p.Hq;
     const int b = (int)(lb % p.B), layer = (int)(lb / p.B);
-    const int len = min(p.lens[b], p.max_chunks * p.chunk_len);
-    const int n_chunks = (len + p.chunk_len - 1) / p.chunk_len;
-    if (n_chunks == 1) return;  // written by the split kernel
+    const int len = seq_keys(p, p.lens[b], p.kv_start[b]);
+    // pieces 0 .. n - 1; the slot of piece c is slot0 (c = 0) or slot1 + c * step
+    int n = (len + p.chunk_len - 1) / p.chunk_len;
+    int64_t slot0 = unit * p.max_chunks, slot1 = slot0, step = 1;
+    if (p.groups > 0 && len > 0) {
+        int before = 0, sum = 0;
+        for (int i = lane; i < p.B; i += 32) {
+            const int li = seq_keys(p, p.lens[i], p.kv_start[i]);
+            sum += li;
+            before += i < b ? li : 0;
+        }
+        sum = __reduce_add_sync(0xffffffffu, sum);
+        before = __reduce_add_sync(0xffffffffu, before);
+        const int per = share_of(sum * n_layers, p.groups), s0 = layer * sum + before;
+        // first and last group with keys of this sequence: its cuts are those of the
+        // multiples of per in [s0, s0 + len)
+        const int lo = (s0 + per - 1) / per, hi = (s0 + len - 1) / per;
+        const int ga = lo <= hi && snap(lo * per - s0, len) == 0 ? lo : lo - 1;
+        const int gz = lo <= hi && snap(hi * per - s0, len) == len ? hi - 1 : hi;
+        const int heads = p.slot_heads, kvh = h / heads, hl = h % heads;
+        n = gz - ga + 1;
+        slot0 = (((int64_t)ga * p.Hkv + kvh) * 2 + 1) * heads + hl;  // from the sequence's start
+        step = (int64_t)p.Hkv * 2 * heads;
+        slot1 = slot0 - heads;
+    }
+    if (n == 1) return;  // written by the split kernel
     uint16_t *op = p.O + layer * p.o_ls + ((int64_t)b * p.Hq + h) * D;
     constexpr int kDpl = D / 32;
-    if (n_chunks <= 0) {
+    using Vec = typename std::conditional<kDpl == 4, float4, float2>::type;
+    if (n <= 0) {
 #pragma unroll
         for (int e = 0; e < kDpl; ++e) op[lane * kDpl + e] = 0;
         if (lane == 0 && p.lse != nullptr) p.lse[unit] = -INFINITY;
         if (lane == 0 && p.nexus_mass != nullptr) p.nexus_mass[unit] = 0.f;
         return;
     }
-    const float *ml = p.part_ml + unit * p.max_chunks * 2;
-    const float *ac = p.part_acc + unit * p.max_chunks * D;
-    float M = -INFINITY;
-    for (int c = lane; c < n_chunks; c += 32) M = fmaxf(M, ml[2 * c]);
+    auto slot_of = [&](int c) { return c == 0 ? slot0 : slot1 + c * step; };
+    const float2 *mls = reinterpret_cast<const float2 *>(p.part_ml);
+    auto acc_of = [&](int c) {
+        return reinterpret_cast<const Vec *>(p.part_acc + slot_of(c) * D)[lane];
+    };
+    // the first pieces' accumulators and every lane's first (max, sum): one round trip
+    constexpr int kFirst = 8;
+    Vec first[kFirst];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+    for (int c = 0; c < kFirst; ++c)
+        if (c < n) first[c] = acc_of(c);
+    float2 ml = make_float2(-INFINITY, 0.f);
+    if (lane < n) ml = mls[slot_of(lane)];
+    float M = ml.x;
+    for (int c = lane + 32; c < n; c += 32) M = fmaxf(M, mls[slot_of(c)].x);
+    M = warp_max(M);
     float L = 0.f, N = 0.f;
     float a[kDpl];
 #pragma unroll
     for (int e = 0; e < kDpl; ++e) a[e] = 0.f;
-    for (int c = 0; c < n_chunks; ++c) {
-        const float f = ex2(ml[2 * c] - M);
-        L += f * ml[2 * c + 1];
-        if (p.nexus_mass != nullptr) N += f * p.part_nx[unit * p.max_chunks + c];
+    for (int c0 = 0; c0 < n; c0 += 32) {
+        float n_l = 0.f;
+        if (c0 + lane < n) {
+            if (c0 > 0) ml = mls[slot_of(c0 + lane)];
+            if (p.nexus_mass != nullptr) n_l = p.part_nx[slot_of(c0 + lane)];
+        }
+        const float f_l = c0 + lane < n ? ex2(ml.x - M) : 0.f;
+        auto add = [&](int c, const Vec &v) {
+            const float f = __shfl_sync(0xffffffffu, f_l, c);
+            L += f * __shfl_sync(0xffffffffu, ml.y, c);
+            N += f * __shfl_sync(0xffffffffu, n_l, c);
+            const float *vp = reinterpret_cast<const float *>(&v);
 #pragma unroll
-        for (int e = 0; e < kDpl; ++e) a[e] += f * ac[(int64_t)c * D + lane * kDpl + e];
+            for (int e = 0; e < kDpl; ++e) a[e] += f * vp[e];
+        };
+        int c = 0;
+        if (c0 == 0) {
+#pragma unroll
+            for (int k = 0; k < kFirst; ++k)
+                if (k < n) add(k, first[k]);
+            c = kFirst;
+        }
+        const int m = min(n - c0, 32);
+#pragma unroll 8
+        for (; c < m; ++c) add(c, acc_of(c0 + c));
     }
+    uint32_t w[kDpl / 2];
 #pragma unroll
-    for (int e = 0; e < kDpl; ++e)
-        op[lane * kDpl + e] = __bfloat16_as_ushort(__float2bfloat16_rn(a[e] / L));
+    for (int e = 0; e < kDpl / 2; ++e) w[e] = pack_bf16x2(a[2 * e] / L, a[2 * e + 1] / L);
+#pragma unroll
+    for (int e = 0; e < kDpl; ++e) op[lane * kDpl + e] = (uint16_t)(w[e >> 1] >> ((e & 1) * 16));
     if (lane == 0 && p.lse != nullptr) p.lse[unit] = (M + __log2f(L)) * kLn2;
     if (lane == 0 && p.nexus_mass != nullptr) p.nexus_mass[unit] = N / L;
 }
@@ -781,6 +947,7 @@ int g_template(int G) {
 
 struct Plan {
     int chunk_len, max_chunks;
+    int groups;  // > 0: equal shares
     // partial accumulators, partial (max, sum), partial Nexus sums, unit counter
     size_t ws_acc, ws_ml, ws_nx, ws_cnt;
     size_t total() const { return ws_acc + ws_ml + ws_nx + ws_cnt; }
@@ -795,7 +962,7 @@ bool use_pairs(const sonic_decode_args *a) {
 
 Plan make_plan(const sonic_decode_args *a) {
     Plan pl{};
-    const int kv_units = a->n_heads_kv / (use_pairs(a) ? 2 : 1);  // KV heads (or pairs) per unit row
+    const int kv_units = a->n_heads_kv < 1 ? 1 : a->n_heads_kv / (use_pairs(a) ? 2 : 1);  // KV heads (or pairs) per unit row
     const int max_len = a->max_len > 0 ? a->max_len : 1;
     // explicit split lengths are rounded up to the kernel's key tile
     const int tile = kTcKeys;
@@ -812,12 +979,19 @@ Plan make_plan(const sonic_decode_args *a) {
     pl.chunk_len = C;
     pl.max_chunks = (max_len + C - 1) / C;
     const size_t units_q = (size_t)a->batch * a->n_heads_q * a->n_layers;
-    if (pl.max_chunks > 1) {
-        pl.ws_acc = round_up(units_q * pl.max_chunks * a->head_dim * sizeof(float), 256);
-        pl.ws_ml = round_up(units_q * pl.max_chunks * 2 * sizeof(float), 256);
-        if (a->nexus_mass != nullptr)
-            pl.ws_nx = round_up(units_q * pl.max_chunks * sizeof(float), 256);
+    size_t slots = pl.max_chunks > 1 ? units_q * pl.max_chunks : 0;
+    const int sms = device_sm_count();
+    const long long keys = (long long)a->n_layers * a->batch * pl.max_chunks * C;
+    if (a->chunk_len == 0 && a->batch <= TcCfg::kSeqCache && kv_units >= 1 && kv_units <= sms &&
+        sms / kv_units * kv_units * 8 >= sms * 7 && keys <= (1 << 30)) {
+        const long long most = (keys + kMinShare - 1) / kMinShare;
+        pl.groups = (int)(most < sms / kv_units ? most : sms / kv_units);
+        // two partial pieces per block, of all query heads of its unit
+        slots = (size_t)pl.groups * kv_units * 2 * (a->n_heads_q / kv_units);
     }
+    pl.ws_acc = round_up(slots * a->head_dim * sizeof(float), 256);
+    pl.ws_ml = round_up(slots * 2 * sizeof(float), 256);
+    if (a->nexus_mass != nullptr) pl.ws_nx = round_up(slots * sizeof(float), 256);
     pl.ws_cnt = 256;  // the persistent kernel's unit counter
     return pl;
 }
@@ -837,6 +1011,9 @@ cudaError_t launch_tc(const TcMaps &m, const DecParams &p, int units_x, int n_un
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
+    if (p.groups > 0)
+        return launch_pdl(kern, dim3(p.groups * p.Hkv), kTcThreads, smem, stream, 1, m.k, m.v, m.q,
+                          m.k16, m.v16, p, units_x, n_units, counter);
     e = cudaMemsetAsync(counter, 0, sizeof(int), stream);
     if (e != cudaSuccess) return e;
     const int sms = device_sm_count();
@@ -969,6 +1146,10 @@ extern "C" sonic_status_t sonic_attn_decode(const uint16_t *q, const uint16_t *K
     p.o_ls = a->o_layer_stride;
     p.chunk_len = pl.chunk_len;
     p.max_chunks = pl.max_chunks;
+    p.n_layers = a->n_layers;
+    p.groups = pl.groups;
+    p.slot_heads = pairs ? 2 * G : G;
+    p.slot_stride = pl.groups > 0 ? 1 : pl.max_chunks;
     const float scale = a->softmax_scale > 0.f ? a->softmax_scale : 1.0f / sqrtf((float)D);
     p.scale_log2 = scale * kLog2e;
 
@@ -983,9 +1164,7 @@ extern "C" sonic_status_t sonic_attn_decode(const uint16_t *q, const uint16_t *K
     if (e != cudaSuccess) return SONIC_ERR_CUDA;
     const long long units = (long long)a->n_layers * a->batch * a->n_heads_q;
     const unsigned cblocks = (unsigned)((units * 32 + 127) / 128);
-    if (D == 128)
-        decode_combine_kernel<128><<<cblocks, 128, 0, stream>>>(p, a->n_layers);
-    else
-        decode_combine_kernel<64><<<cblocks, 128, 0, stream>>>(p, a->n_layers);
-    return cudaGetLastError() == cudaSuccess ? SONIC_OK : SONIC_ERR_CUDA;
+    e = launch_pdl(D == 128 ? decode_combine_kernel<128> : decode_combine_kernel<64>, dim3(cblocks),
+                   128, 0, stream, 1, p, a->n_layers);
+    return e == cudaSuccess ? SONIC_OK : SONIC_ERR_CUDA;
 }

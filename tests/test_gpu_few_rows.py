@@ -4,8 +4,12 @@ of its row paddings (16, 32, 64, 128, 192), with and without a split, ragged col
 tiles, one kind of row or both."""
 import numpy as np
 import pytest
+import torch
 
-from paper_2601_21927_gb300 import inputs
+from paper_2601_21927_gb300 import inputs, sonic
+from tests import harness as H
+from tests.test_gpu_decode import _check as _check_decode
+from tests.test_gpu_decode import _check_mass, _decode
 from tests.test_gpu_routed import _check, _roles, _run
 
 pytestmark = pytest.mark.gpu
@@ -28,3 +32,56 @@ def test_routed_linear_projection_widths(role, T, d_in, cols):
     roles = _roles(T, T) if role is None else np.full(T, role, np.uint8)
     r = _run(roles, d_in, cols, [False] + [True] * (len(cols) - 1), seed=41, cache_rows=T + 9)
     _check(r)
+
+
+@pytest.mark.parametrize("hq,hkv,D,nl", [(32, 8, 128, 1), (28, 4, 128, 3), (4, 2, 64, 2),
+                                         (3, 1, 128, 1), (16, 1, 64, 1), (30, 15, 128, 1)])
+@pytest.mark.parametrize("lens", [
+    [1], [16], [63, 64, 65], [128 * 19 + 31], [0, 5, 0, 700, 0], [4096, 1, 33, 31, 32, 2050],
+    list(range(1, 130))], ids=lambda v: f"{len(v)}x{max(v)}")
+def test_decode_equal_shares(lens, hq, hkv, D, nl):
+    """Sequences shorter than a share, far longer, empty, ending next to a cut (within the
+    32 keys a cut moves by), many to a block; lse and Nexus mass too."""
+    r = _decode(np.array(lens, np.int32), hq, hkv, D, n_layers=nl, seed=len(lens) + hq,
+                with_mass=True)
+    pairs = [(nl - 1, b) for b in range(0, len(lens), 1 + len(lens) // 12)] + [(0, len(lens) - 1)]
+    _check_decode(r, pairs)
+    _check_mass(r, pairs)
+    assert not r["O"].isnan().any()
+
+
+def test_calls_captured_after_copies_and_memsets():
+    """A graph whose calls follow a copy and a memset (no kernel before them): replays equal
+    the eager calls bit for bit."""
+    lens, starts = H.i32([700, 45]), H.i32([0, 700])
+    K = inputs.randn((1, 745, 8, 128), seed=1, device=H.dev())
+    V = inputs.randn((1, 745, 8, 128), seed=2, device=H.dev())
+    q = inputs.randn((1, 2, 32, 128), seed=3, device=H.dev())
+    W = inputs.randn((256, 4096), seed=4, device=H.dev())
+    role = torch.full((2,), inputs.ROLE_CURR, dtype=torch.uint8, device=H.dev())
+    qc, O = torch.empty_like(q), torch.empty_like(q)
+    Y = torch.empty((2, 256), dtype=torch.bfloat16, device=H.dev())
+    z = torch.empty(1 << 20, device=H.dev())
+
+    def step(ws):
+        z.zero_()
+        qc.copy_(q)
+        w0 = sonic.sonic_attn_decode(qc, K, V, lens, O, kv_start=starts, max_len=700,
+                                     workspace=ws[0])
+        z.zero_()
+        return w0, sonic.sonic_routed_linear(O.view(2, 4096), W, W, role, [(Y, False)],
+                                             workspace=ws[1])
+
+    ws = step((None, None))
+    torch.cuda.synchronize()
+    want = O.clone(), Y.clone()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        step(ws)
+    for _ in range(3):
+        O.fill_(float("nan"))
+        Y.fill_(float("nan"))
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(O.view(torch.int16), want[0].view(torch.int16))
+        assert torch.equal(Y.view(torch.int16), want[1].view(torch.int16))
