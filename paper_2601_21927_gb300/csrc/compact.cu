@@ -5,7 +5,10 @@
 // effective context is I_sys + Nexus state + current query): a row is kept
 // iff its role is not BODY; kept rows keep their order.
 //
-// Four launches, none of which needs a host round trip:
+// Launches, none of which needs a host round trip.  Calls of up to 524,288 rows:
+//   keep_plan     the whole scan in one launch (see there);
+//   kv_gather     below.
+// Larger calls:
 //   keep_count    one block per (chunk, sequence), each sequence cut into
 //                 kChunks pieces: kept rows of the piece (and a layout check
 //                 when segment numbers are given);
@@ -18,6 +21,9 @@
 //                 rows);
 //   kv_gather     all layers, K and V: 16-byte vector copy of every kept row
 //                 to its output row, grid-stride over rows of each layer.
+#include <algorithm>
+#include <climits>
+
 #include "sonic_dev.cuh"
 #include "sonic_host.h"
 
@@ -26,6 +32,12 @@ namespace {
 
 constexpr int kScanThreads = 512;
 constexpr int kChunks = 64;  // pieces per sequence in the scans
+// the single-launch scan (keep_plan): its largest call (rows; rows x sequences, which
+// bounds what a block counts where sequences share rows), and rows per piece
+constexpr int kPlanRows = 1 << 19;
+constexpr int64_t kPlanWork = 1 << 25;
+constexpr int kPlanRowsPerThread = 4;
+constexpr int kPlanStep = kScanThreads * kPlanRowsPerThread;  // rows per piece, mostly
 
 // Rows of sequence (start, len), or 0 when they fall outside [0, total): such a
 // sequence is refused, keeps nothing and is never read.
@@ -192,6 +204,164 @@ keep_scatter_kernel(const uint8_t *__restrict__ role, const int32_t *__restrict_
     }
 }
 
+// Kept rows among n role bytes at p, this thread's share: thread `lane` of `lanes`
+// (>= 16) takes 16-byte words lane, lane + lanes, ... between the unaligned ends.
+__device__ __forceinline__ int count_kept(const uint8_t *p, int n, int lane, int lanes) {
+    const int head = min(n, (int)((16 - (reinterpret_cast<uintptr_t>(p) & 15)) & 15));
+    const int words = (n - head) >> 4, tail = (n - head) & 15;
+    int kept = lane < head && p[lane] != SONIC_ROLE_BODY;
+    kept += lane < tail && p[n - tail + lane] != SONIC_ROLE_BODY;
+    const uint4 *w = reinterpret_cast<const uint4 *>(p + head);
+    constexpr uint32_t kBody4 = 0x01010101u * SONIC_ROLE_BODY;
+#pragma unroll 8
+    for (int i = lane; i < words; i += lanes) {
+        const uint4 v = w[i];
+        kept += 16 - (__popc(__vcmpeq4(v.x, kBody4)) + __popc(__vcmpeq4(v.y, kBody4)) +
+                      __popc(__vcmpeq4(v.z, kBody4)) + __popc(__vcmpeq4(v.w, kBody4))) / 8;
+    }
+    return kept;
+}
+
+// keep_count, keep_bases and keep_scatter in one launch, for calls of at most
+// kPlanRows rows: every block counts the kept rows before its own piece itself, from
+// the role bytes (16 per load, out of L2; one run where the sequences are packed), so no
+// block waits for another and nothing is exchanged between launches.  Bound by its chain
+// of dependent loads (lengths, role bytes, then the writes): 5.5 us alone for one
+// sequence of 2,688 rows, 8.9 us for 8 ragged ones (~90k rows), 16 us for 64 (~450k
+// rows), where every block reads 225 KB on average.  The three launches it replaces
+// made the whole call (GPU time, us, three launches / this) 60.2 / 53.9 for one
+// sequence of 100k rows, 95.5 / 78.7 for 32 of 3k, 212 / 185 for 64 of 4k and 71.3 / 69.4 for two
+// of 250k: the line lies where the gain has run out (the counted bytes grow with the
+// square of the rows).
+// blockIdx = (piece, sequence); gridDim.x pieces per sequence.
+__global__ void __launch_bounds__(kScanThreads)
+keep_plan_kernel(const uint8_t *role, const int32_t *seg,
+                 const int32_t *k_start, const int32_t *k_len,
+                 const int32_t *reserve, int32_t B, int32_t capacity, int32_t total,
+                 int32_t *offsets, int32_t *ret_len,
+                 int32_t *src_idx, uint8_t *out_role,
+                 int32_t *out_seg, int32_t *status) {
+    pdl_wait();
+    pdl_trigger();
+    const int c = blockIdx.x, b = blockIdx.y, pieces = gridDim.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr int kWarps = kScanThreads / 32;
+    __shared__ long long seq_part[kWarps];
+    __shared__ int own_part[kWarps], warp_tot[kWarps];
+    const int32_t start = k_start[b], len_in = k_len[b], first = k_start[0];
+    // sequences packed one after another (as a batch's mostly are) are counted as one run
+    bool packed = true;
+    long long before = 0;
+    for (int i = tid; i < b; i += kScanThreads) {
+        const int32_t s = k_start[i], n = k_len[i];
+        packed = packed && s >= 0 && n >= 0 && (int64_t)s + n <= total && s + n == k_start[i + 1];
+        if (reserve != nullptr) before += reserve[i];
+    }
+    const int32_t len = seq_rows(start, len_in, total);
+    if (c == 0 && tid == 0 && len != len_in) set_status(status, SONIC_ERR_INVALID_ARGUMENT);
+    const int32_t rows = ((len + pieces - 1) / pieces + 31) & ~31;
+    const int32_t lo = min(len, c * rows), hi = min(len, lo + rows);
+    // this thread's rows of the piece's first step, loaded ahead of the counts
+    int32_t t0 = lo + tid * kPlanRowsPerThread;
+    int ro[kPlanRowsPerThread], sg[kPlanRowsPerThread + 1];
+    auto load = [&](int32_t t) {
+        sg[0] = seg != nullptr && t > 0 && t < hi ? seg[start + t - 1] : INT_MIN;
+#pragma unroll
+        for (int k = 0; k < kPlanRowsPerThread; ++k) {
+            ro[k] = t + k < hi ? role[start + t + k] : -1;
+            sg[k + 1] = seg != nullptr && t + k < hi ? seg[start + t + k] : 0;
+        }
+    };
+    load(t0);
+    // rows kept (and reserved) by the sequences before this one, and by this sequence's
+    // pieces before this one
+    if (__syncthreads_and(packed)) {
+        if (b > 0) before += count_kept(role + first, start - first, tid, kScanThreads);
+    } else {
+        int wps = kWarps;  // several warps a sequence while there are few
+        while (wps > 1 && wps * b > kWarps) wps >>= 1;
+        for (int i = warp / wps; i < b; i += kWarps / wps) {
+            const int32_t s = k_start[i], n = seq_rows(s, k_len[i], total);
+            before += count_kept(role + s, n, (warp % wps) * 32 + lane, wps * 32);
+        }
+    }
+    int own = count_kept(role + start, lo, tid, kScanThreads);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
+    own = __reduce_add_sync(0xffffffffu, own);
+    if (lane == 0) {
+        seq_part[warp] = before;
+        own_part[warp] = own;
+    }
+    long long seq_base = 0, running = 0;
+    bool bad = false;
+    for (int32_t c0 = lo; c0 == lo || c0 < hi; c0 += kPlanStep) {
+        int n = 0;  // this thread's kept rows
+#pragma unroll
+        for (int k = 0; k < kPlanRowsPerThread; ++k) {
+            const bool in = ro[k] >= 0, body = ro[k] == SONIC_ROLE_BODY;
+            n += in && !body;
+            bad |= ro[k] > SONIC_ROLE_CURR;
+            if (seg != nullptr && in) bad |= (body && sg[k + 1] <= 0) || sg[k + 1] < sg[k];
+        }
+        const int incl = warp_inclusive_scan(n);
+        if (lane == 31) warp_tot[warp] = incl;
+        __syncthreads();
+        if (c0 == lo) {
+#pragma unroll
+            for (int w = 0; w < kWarps; ++w) {
+                seq_base += seq_part[w];
+                running += own_part[w];
+            }
+            running += seq_base;
+        }
+        int warp_base = 0, step_tot = 0;
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) {
+            const int v = warp_tot[w];
+            if (w < warp) warp_base += v;
+            step_tot += v;
+        }
+        long long o = running + warp_base + incl - n;
+#pragma unroll
+        for (int k = 0; k < kPlanRowsPerThread; ++k) {
+            if (ro[k] < 0 || ro[k] == SONIC_ROLE_BODY) continue;
+            if (o < capacity) {
+                src_idx[o] = start + t0 + k;
+                if (out_role) out_role[o] = (uint8_t)ro[k];
+                if (out_seg) out_seg[o] = sg[k + 1];
+            }
+            ++o;
+        }
+        running += step_tot;
+        t0 += kPlanStep;
+        if (c0 + kPlanStep < hi) load(t0);
+        __syncthreads();
+    }
+    if (__syncthreads_or(bad) && tid == 0) set_status(status, SONIC_ERR_LAYOUT);
+    if (c == 0 && tid == 0) offsets[b] = (int32_t)seq_base;
+    if (c != pieces - 1) return;
+    // the sequence's last piece: its retained length, its reserve rows (no source), and
+    // behind the last sequence the total
+    const int32_t res = reserve != nullptr ? reserve[b] : 0;
+    for (int32_t r = tid; r < res; r += kScanThreads) {
+        const long long o = running + r;
+        if (o < capacity) {
+            src_idx[o] = -1;
+            if (out_role) out_role[o] = SONIC_ROLE_BODY;
+            if (out_seg) out_seg[o] = -1;
+        }
+    }
+    if (tid == 0) {
+        if (ret_len) ret_len[b] = (int32_t)(running - seq_base);
+        if (b == B - 1) {
+            offsets[B] = (int32_t)(running + res);
+            if (running + res > capacity || running + res > 0x7fffffffLL)
+                set_status(status, SONIC_ERR_CAPACITY);
+        }
+    }
+}
+
 // 16-byte vector copy of kept rows.  blockIdx.y = layer * 2 + (0: K, 1: V).
 // One warp copies whole rows (lane j takes 16-byte chunks j, j+32, ...); each
 // warp works on two rows at a time with all their loads issued before the
@@ -212,30 +382,37 @@ __device__ __forceinline__ int4 ld_stream(const void *p) {
 // rows in flight helps the long rows; at 1 KB it measured slower).
 template <int kGatherRows, int kGatherUnroll>
 __global__ void __launch_bounds__(kGatherThreads)
-kv_gather_kernel(const uint8_t *__restrict__ K, const uint8_t *__restrict__ V,
-                 uint8_t *__restrict__ out_K, uint8_t *__restrict__ out_V,
-                 const int32_t *__restrict__ offsets, const int32_t *__restrict__ src_idx,
+kv_gather_kernel(const uint8_t *K, const uint8_t *V,
+                 uint8_t *out_K, uint8_t *out_V,
+                 const int32_t *offsets, const int32_t *src_idx,
                  int32_t B, int32_t capacity, int64_t row_bytes, int64_t in_layer_bytes,
                  int64_t out_layer_bytes) {
+    pdl_wait();
+    pdl_trigger();
     const int layer = blockIdx.y >> 1;
     const bool is_v = blockIdx.y & 1;
     const uint8_t *src = (is_v ? V : K) + (int64_t)layer * in_layer_bytes;
     uint8_t *dst = (is_v ? out_V : out_K) + (int64_t)layer * out_layer_bytes;
-    int64_t n_rows = offsets[B];
-    if (n_rows > capacity) n_rows = capacity;
+    const int64_t n_rows = min(offsets[B], capacity);
     const int lane = threadIdx.x & 31;
     const int64_t n_warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     const int cpr = (int)(row_bytes >> 4);  // 16-byte chunks per row
     // each warp moves kGatherRows rows per pass (n_warps apart), every lane
     // holding its 16-byte pieces of all of them in flight
-    for (int64_t r0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5); r0 < n_rows;
+    for (int64_t r0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5); r0 < capacity;
          r0 += kGatherRows * n_warps) {
         int32_t sr[kGatherRows];
 #pragma unroll
         for (int k = 0; k < kGatherRows; ++k) {
+            // (read below the capacity, so that it does not wait for the row count:
+            // 494 -> 476 us on 3.22 GB of 2 KB rows)
             const int64_t r = r0 + k * n_warps;
-            sr[k] = r < n_rows ? src_idx[r] : -1;
+            sr[k] = r < capacity ? src_idx[r] : -1;
         }
+#pragma unroll
+        for (int k = 0; k < kGatherRows; ++k)
+            if (r0 + k * n_warps >= n_rows) sr[k] = -1;
+        if (r0 >= n_rows) break;
         for (int c0 = lane; c0 < cpr; c0 += 32 * kGatherUnroll) {
             int4 v[kGatherRows][kGatherUnroll];
 #pragma unroll
@@ -313,15 +490,27 @@ extern "C" sonic_status_t sonic_compact_kv(const void *K, const void *V, const i
     ws += round_up((size_t)a->batch * sizeof(long long), 256);
     int32_t *src_idx = a->src_idx != nullptr ? a->src_idx : reinterpret_cast<int32_t *>(ws);
 
-    const dim3 pieces(kChunks, a->batch);
-    keep_count_kernel<<<pieces, kScanThreads, 0, stream>>>(role, seg_id, a->k_start, a->k_len,
-                                                          a->total_rows, counts, a->status);
-    keep_bases_kernel<<<1, kScanThreads, 0, stream>>>(counts, a->reserve, a->batch,
-                                                      a->out_capacity_rows, seq_base, offsets,
-                                                      a->ret_len, a->status);
-    keep_scatter_kernel<<<pieces, kScanThreads, 0, stream>>>(
-        role, seg_id, a->k_start, a->k_len, a->reserve, counts, seq_base, a->out_capacity_rows,
-        a->total_rows, src_idx, a->out_role, a->out_seg);
+    cudaError_t e = cudaSuccess;
+    if (a->total_rows <= kPlanRows && (int64_t)a->total_rows * a->batch <= kPlanWork) {
+        const int rows = a->total_rows / a->batch;
+        const int n = std::min(kChunks, std::max(1, (rows + kPlanStep - 1) / kPlanStep));
+        e = launch_pdl(keep_plan_kernel, dim3(n, a->batch), kScanThreads, 0, stream, 1, role, seg_id,
+                       a->k_start, a->k_len, a->reserve, a->batch, a->out_capacity_rows,
+                       a->total_rows, offsets, a->ret_len, src_idx, a->out_role, a->out_seg,
+                       a->status);
+    } else {
+        const dim3 pieces(kChunks, a->batch);
+        keep_count_kernel<<<pieces, kScanThreads, 0, stream>>>(
+            role, seg_id, a->k_start, a->k_len, a->total_rows, counts, a->status);
+        keep_bases_kernel<<<1, kScanThreads, 0, stream>>>(counts, a->reserve, a->batch,
+                                                          a->out_capacity_rows, seq_base, offsets,
+                                                          a->ret_len, a->status);
+        keep_scatter_kernel<<<pieces, kScanThreads, 0, stream>>>(
+            role, seg_id, a->k_start, a->k_len, a->reserve, counts, seq_base, a->out_capacity_rows,
+            a->total_rows, src_idx, a->out_role, a->out_seg);
+        e = cudaGetLastError();
+    }
+    if (e != cudaSuccess) return SONIC_ERR_CUDA;
     const int sms = device_sm_count();
     // ~32 blocks per SM in all (four resident at a time): with many small
     // blocks the SMs run out of work together, where ~8 left a ragged tail
@@ -329,9 +518,9 @@ extern "C" sonic_status_t sonic_compact_kv(const void *K, const void *V, const i
     const int per_slice = (sms * 32 + 2 * a->n_layers - 1) / (2 * a->n_layers);
     dim3 grid(per_slice < 1 ? 1 : per_slice, 2 * a->n_layers);
     auto gather = a->row_bytes >= 2048 ? kv_gather_kernel<4, 2> : kv_gather_kernel<2, 4>;
-    gather<<<grid, kGatherThreads, 0, stream>>>(
-        static_cast<const uint8_t *>(K), static_cast<const uint8_t *>(V),
-        static_cast<uint8_t *>(out_K), static_cast<uint8_t *>(out_V), offsets, src_idx, a->batch,
-        a->out_capacity_rows, a->row_bytes, a->in_layer_bytes, a->out_layer_bytes);
-    return cudaGetLastError() == cudaSuccess ? SONIC_OK : SONIC_ERR_CUDA;
+    e = launch_pdl(gather, grid, kGatherThreads, 0, stream, 1, static_cast<const uint8_t *>(K),
+                   static_cast<const uint8_t *>(V), static_cast<uint8_t *>(out_K),
+                   static_cast<uint8_t *>(out_V), offsets, src_idx, a->batch,
+                   a->out_capacity_rows, a->row_bytes, a->in_layer_bytes, a->out_layer_bytes);
+    return e == cudaSuccess ? SONIC_OK : SONIC_ERR_CUDA;
 }

@@ -160,7 +160,9 @@ __device__ __forceinline__ bool mbar_drain(uint64_t *bar, uint32_t parity) {
 // calls pdl_wait() before it touches global memory: it returns once all earlier
 // kernels of the stream have completed and their writes are visible.
 // pdl_trigger() lets the kernel after this one start its own set-up early; that
-// one waits the same way, so it is safe at any point.
+// one waits the same way, so it is safe at any point.  Pointers that such a kernel
+// reads through are not __restrict__ const: a load the compiler takes for invariant
+// could be moved above the wait.
 
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

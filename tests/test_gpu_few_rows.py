@@ -8,6 +8,8 @@ import torch
 
 from paper_2601_21927_gb300 import inputs, sonic
 from tests import harness as H
+from tests.test_gpu_compact import _check as _check_compact
+from tests.test_gpu_compact import _run as _compact
 from tests.test_gpu_decode import _check as _check_decode
 from tests.test_gpu_decode import _check_mass, _decode
 from tests.test_gpu_routed import _check, _roles, _run
@@ -85,3 +87,30 @@ def test_calls_captured_after_copies_and_memsets():
         torch.cuda.synchronize()
         assert torch.equal(O.view(torch.int16), want[0].view(torch.int16))
         assert torch.equal(Y.view(torch.int16), want[1].view(torch.int16))
+
+
+@pytest.mark.parametrize("n_seqs,rows,total", [(1, 131072, 131072), (1, 131073, 131073),
+                                               (2, 2047, 0), (3, 2049, 0), (15, 900, 0),
+                                               (17, 4100, 0), (40, 77, 0), (128, 300, 0)])
+def test_compact_single_launch_scan(n_seqs, rows, total):
+    """On both sides of the largest call of the single-launch scan (131,072 rows), sequences
+    at every alignment of the role bytes, pieces that end off the 16-byte words, empty
+    and body-only sequences among them, reserve rows."""
+    rng = np.random.default_rng(rows)
+    ds = []
+    for k in range(n_seqs):
+        n = total // n_seqs if total else int(rng.integers(1, rows + 1))
+        segs, left = [], n
+        while left > 700:
+            b, x = int(rng.integers(0, 600)), int(rng.integers(0, 70))
+            segs.append((b, x))
+            left -= b + x
+        ds.append(inputs.Dialogue(int(rng.integers(0, left + 1)) if not total else left, segs, 0))
+    if n_seqs > 2:
+        ds[1], ds[2] = inputs.Dialogue(0, [], 0), inputs.Dialogue(0, [(333, 0)], 0)
+    batch = inputs.Batch(ds)
+    assert not total or batch.total == total
+    K = inputs.randn((1, batch.total, 1, 8), seed=rows, device=H.dev())
+    V = inputs.randn((1, batch.total, 1, 8), seed=rows + 1, device=H.dev())
+    reserve = rng.integers(0, 5, batch.B)
+    _check_compact(batch, K, V, _compact(batch, K, V, reserve=reserve), reserve=reserve)
