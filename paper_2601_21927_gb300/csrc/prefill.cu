@@ -28,6 +28,7 @@
 // a block overlap: the next unit's first S products run while the softmax
 // warps finish the previous one.
 #include <algorithm>
+#include <atomic>
 #include <cstddef>
 #include <type_traits>
 
@@ -101,7 +102,8 @@ struct PfParams {
     int32_t *status;
     const TileSum *sums;
     const TileMasks *masks;  // per key tile, from the summary kernel
-    int32_t *counter;        // next work unit to claim (zeroed by the summary kernel)
+    int32_t *counter;        // next work unit to claim (set by the summary kernel)
+    int n_split;             // kSplit: blocks per unit
     int n_units, qtiles, HG; // units = qtiles x HG x B x n_layers; HG = Hq >> pack_log2
     int max_k_tiles, max_k_len;
     int B, Hq, G;
@@ -298,14 +300,17 @@ __device__ __forceinline__ void build_tile_masks(const int (&ro)[4], const int (
 }
 
 __global__ void __launch_bounds__(128)
-tile_summary_kernel(const uint8_t *__restrict__ role, const int32_t *__restrict__ seg,
-                    const int32_t *__restrict__ pos, const int32_t *__restrict__ k_start,
-                    const int32_t *__restrict__ k_len, TileSum *__restrict__ out,
-                    TileMasks *__restrict__ masks_out, int max_k_tiles, int64_t total_rows,
-                    int32_t *status, int32_t *unit_counter) {
+tile_summary_kernel(const uint8_t *role, const int32_t *seg,
+                    const int32_t *pos, const int32_t *k_start,
+                    const int32_t *k_len, TileSum *out,
+                    TileMasks *masks_out, int max_k_tiles, int64_t total_rows,
+                    int32_t *status, int32_t *unit_counter, int first_claim) {
+    pdl_wait();
+    pdl_trigger();
     const int t = blockIdx.x, b = blockIdx.y;
-    // the attention kernel that follows claims its work units from 0
-    if (t == 0 && b == 0 && threadIdx.x == 0) *unit_counter = 0;
+    // the attention kernel's blocks start with the units of their own indices and claim
+    // the others from there (chunked query order: claim every unit, from 0)
+    if (t == 0 && b == 0 && threadIdx.x == 0) *unit_counter = first_claim;
     const int len_in = k_len[b];
     // a sequence outside the arrays (or longer than the tiles) gets empty summaries
     const int len = seq_rows(k_start[b], len_in, max_k_tiles * kBN, total_rows);
@@ -508,7 +513,14 @@ __device__ __forceinline__ void tile_mask_bits(const TileMasks *tmk, const uint8
 // three stages (the unused second Q tile's buffer is the third), V of two.
 // kPair: paired units (an even number of query heads per KV head, heads not
 // packed): a unit is one 128-row query block of heads h0 and h0 + 1.
-template <int D, int kOut, bool kQC, bool kSolo, bool kPair>
+// kSplit: calls of few units.  A cluster of S blocks shares one unit (block index / S,
+// no counter), each taking every S-th of its listed key tiles, and the blocks merge
+// their partial rows (log-sum-exp, fp32) through distributed shared memory.  Such a call
+// is bound by its longest unit, a chain of ~3.4k clocks per key tile, while most SMs
+// have none: a turn of 333 rows over 2,189 keys (48 units of 17 tiles, S = 2) went from
+// 38 to 29 us, one over 8.7k keys from 126 to 74, 16 rows over 1,872 keys (8 packed
+// units, S = 7) from 22 to 16, the merge among it (~3 us at S = 2, ~5 at S = 7).
+template <int D, int kOut, bool kQC, bool kSolo, bool kPair, bool kSplit>
 __global__ void __maxnreg__(168)
 prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmK0,
@@ -551,7 +563,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     uint64_t *k_empty = bars + 26;  // [3]
     uint64_t *pv_done = bars + 29;
     int32_t *misc = reinterpret_cast<int32_t *>(smem + C::kOffMisc);
-    // misc: 0 tmem base, 2 abort
+    // misc: 0 tmem base, 2 abort, 3 the scheduler copied the first unit's Q
     volatile int *abort_flag = reinterpret_cast<volatile int *>(misc + 2);
 
     // A query tile is R query rows x P heads of one KV group (P = 1 << pack_log2,
@@ -561,6 +573,11 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     // query rows of a unit, and the row offset of its second query tile
     const int urows = kPair ? R : 2 * R, qstep = kPair ? 0 : R;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int n_split = kSplit ? p.n_split : 1, rank = kSplit ? (int)cluster_rank() : 0;
+    // kSplit: (max, sum, unrounded sum, Nexus sum) of each row, and its O in 16-byte
+    // pieces [D / 4][128 rows] per query tile, over the Q and K/V buffers
+    float4 *split_ml = reinterpret_cast<float4 *>(Qs);
+    float4 *split_o = reinterpret_cast<float4 *>(Ks);
 
     if (tid == 0) {
         mbar_init(q_full, 1);
@@ -586,21 +603,42 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
             mbar_init(pv_done, 1);
         }
         *abort_flag = 0;
+        if (!kQC) misc[3] = 0;
         fence_mbar_init();
+        if (!kQC) {
+            tma_prefetch_desc(&tmQ);
+            tma_prefetch_desc(&tmK);
+            tma_prefetch_desc(&tmV);
+            if (p.key_direct != nullptr) {
+                tma_prefetch_desc(&tmK0);
+                tma_prefetch_desc(&tmV0);
+            }
+        }
     }
     if (warp == 1) {
         tmem_alloc(reinterpret_cast<uint32_t *>(&misc[0]), 512);
         tmem_relinquish();
     }
+    if (kQC) pdl_wait();
+    pdl_trigger();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = static_cast<uint32_t>(misc[0]);
+    // The summary kernel before this one lets it start once everything ahead of the call is
+    // complete, so the caller's tensors may be read at once: the scheduler warp starts on the
+    // block's first unit (its own index, no claim) and copies its Q while the summaries
+    // are still being written: a call's first product then starts ~3 us earlier (it came
+    // 8 us after the launch; the tiny dialogue's call took 14.5 us, now 11.6).  Everything else waits for them.  (kQC keeps the plain
+    // order: the same start there made the key-tile loops compile 3-7 % slower.)
+    if (!kQC && warp != kSchedWarp) pdl_wait();
     // what the producer issued, for the drain after an abort
     int issued_q = 0, issued_kv = 0, issued_k = 0;
 
     if (warp == kSchedWarp) {
         // ------------------------------------------------------------ scheduler
+        bool taken = false;  // the block's first unit is taken
+        bool waited = kQC;   // the kernel before this one is complete
         for (int k = 0;; ++k) {
             const int slot = k & 1;
             int end = 0, layer = 0, b = 0, hg = 0, qt = 0, cw = 0;
@@ -608,8 +646,20 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
             int kstart = 0, klen = 0, qstart = 0, qlen = 0, kkstart = 0, kklen = 0;
             for (;;) {
                 int u = p.n_units;
-                if (lane == 0 && !*abort_flag && !timed_out(p.status)) u = atomicAdd(p.counter, 1);
-                u = __shfl_sync(0xffffffffu, u, 0);
+                bool dead = false;
+                if constexpr (kQC) {
+                    if (lane == 0 && !*abort_flag && !timed_out(p.status)) u = atomicAdd(p.counter, 1);
+                    u = __shfl_sync(0xffffffffu, u, 0);
+                } else if (!taken) {
+                    u = kSplit ? blockIdx.x / n_split : blockIdx.x;
+                    dead = timed_out(p.status);  // (tested below, beside the loads that follow)
+                    taken = true;
+                } else if (!kSplit) {
+                    if (!waited) pdl_wait();
+                    waited = true;
+                    if (lane == 0 && !*abort_flag && !timed_out(p.status)) u = atomicAdd(p.counter, 1);
+                    u = __shfl_sync(0xffffffffu, u, 0);
+                }
                 if (u >= p.n_units) {
                     end = 1;
                     break;
@@ -628,6 +678,10 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                 qlen = p.q_len[b];
                 kstart = p.k_start[b];
                 qstart = p.q_start[b];
+                if (!kQC && __shfl_sync(0xffffffffu, dead, 0)) {
+                    end = 1;
+                    break;
+                }
                 if (kstart < 0 || (int64_t)kstart + klen > p.total_k_rows || qstart < 0 ||
                     qlen < 0 || (int64_t)qstart + qlen > p.total_q_rows) {
                     // rows outside the arrays: the sequence is refused, nothing is read
@@ -740,40 +794,61 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                 tile1 = kPair || qp0[1] <= qp1[1];
             } else {
                 tile1 = kPair || (!kPair && lpair) || qt * 2 * R + R < qlen;
+                const int step1 = lpair ? 0 : qstep;
+                // every row's role and segment loaded before any is used
+                int ro[2][kBM / 32], sg[2][kBM / 32];
 #pragma unroll
-                for (int qi = 0; qi < 2; ++qi) {
+                for (int qi = 0; qi < (kPair || kSolo ? 1 : 2); ++qi)
+#pragma unroll
+                    for (int x = 0; x < kBM / 32; ++x) {
+                        const int pos = pbase + qi * step1 + x * 32 + lane;
+                        const bool in = x * 32 + lane < R && pos <= klen - 1;
+                        ro[qi][x] = in ? p.role[kstart + pos] : -1;
+                        sg[qi][x] = in ? p.seg[kstart + pos] : 0;
+                    }
+                if (k == 0 && lane == 0) {
+                    const int nq = tile1 ? 2 : 1, h0 = kPair ? 2 * hg : hg << pl2;
+                    misc[3] = 1;
+                    mbar_arrive_expect_tx(q_full, nq * C::kQBytes);
+                    for (int qi = 0; qi < nq; ++qi)
+                        tma_load_5d(Qs + qi * C::kQBytes, &tmQ, q_full, 0,
+                                    h0 + qi * (kPair ? 1 : (int)lpair),
+                                    qstart + qt * urows + qi * step1, 0, layer);
+                }
+#pragma unroll
+                for (int qi = 0; qi < (kPair || kSolo ? 1 : 2); ++qi) {
                     int f = 0, s0 = INT_MAX, s1 = INT_MIN, n0 = INT_MAX, n1 = INT_MIN;
-                    for (int r = lane; r < R; r += 32) {
-                        const int pos = pbase + qi * (lpair ? 0 : qstep) + r;
-                        if (pos <= klen - 1) {
-                            const int ro = p.role[kstart + pos];
-                            const int s = p.seg[kstart + pos];
-                            s0 = min(s0, s);
-                            s1 = max(s1, s);
-                            if (ro == SONIC_ROLE_NEXUS) {
-                                f = 2;
-                                n0 = min(n0, s);
-                                n1 = max(n1, s);
-                            }
+#pragma unroll
+                    for (int x = 0; x < kBM / 32; ++x) {
+                        if (ro[qi][x] < 0) continue;
+                        s0 = min(s0, sg[qi][x]);
+                        s1 = max(s1, sg[qi][x]);
+                        if (ro[qi][x] == SONIC_ROLE_NEXUS) {
+                            f = 2;
+                            n0 = min(n0, sg[qi][x]);
+                            n1 = max(n1, sg[qi][x]);
                         }
                     }
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) {
-                        f |= __shfl_xor_sync(0xffffffffu, f, o);
-                        s0 = min(s0, __shfl_xor_sync(0xffffffffu, s0, o));
-                        s1 = max(s1, __shfl_xor_sync(0xffffffffu, s1, o));
-                        n0 = min(n0, __shfl_xor_sync(0xffffffffu, n0, o));
-                        n1 = max(n1, __shfl_xor_sync(0xffffffffu, n1, o));
-                    }
-                    qf[qi] = f;
-                    qs0[qi] = s0;
-                    qs1[qi] = s1;
-                    qn0[qi] = n0;
-                    qn1[qi] = n1;
-                    qp0[qi] = pbase + qi * (lpair ? 0 : qstep);
+                    qf[qi] = __reduce_or_sync(0xffffffffu, f);
+                    qs0[qi] = __reduce_min_sync(0xffffffffu, s0);
+                    qs1[qi] = __reduce_max_sync(0xffffffffu, s1);
+                    qn0[qi] = __reduce_min_sync(0xffffffffu, n0);
+                    qn1[qi] = __reduce_max_sync(0xffffffffu, n1);
+                    qp0[qi] = pbase + qi * step1;
                     qp1[qi] = min(qp0[qi] + R - 1, klen - 1);
                 }
+                if (kPair || kSolo) {  // the same rows twice, or (kSolo) no second tile
+                    qf[1] = qf[0];
+                    qs0[1] = qs0[0];
+                    qs1[1] = qs1[0];
+                    qn0[1] = qn0[0];
+                    qn1[1] = qn1[0];
+                    qp0[1] = kSolo ? INT_MAX : qp0[0];
+                    qp1[1] = kSolo ? INT_MIN : qp1[0];
+                }
             }
+            if (!waited) pdl_wait();
+            waited = true;
             // Key tiles to visit: a key tile is listed when either query tile
             // sees some of it.  entry: (tile << 6) | (Nexus keys: 0 none, 1 all,
             // 2 some) << 4 | (tile 1 sees it) << 3 | (tile 0 sees it) << 2
@@ -781,12 +856,16 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
             int32_t *lst = lists + slot * kMaxKTiles;
             const int n_kt = (kklen + kBN - 1) / kBN;
             int n_list = 0, last0 = -1, last1 = -1, skipped = 0;
+            TileSum next{};  // loaded a step ahead (kQC: when needed)
+            if (!kQC && lane < n_kt) next = p.sums[(int64_t)b * p.max_k_tiles + lane];
             for (int c0 = 0; c0 < n_kt; c0 += 32) {
                 const int t = c0 + lane;
+                const TileSum cur = next;
+                if (!kQC && t + 32 < n_kt) next = p.sums[(int64_t)b * p.max_k_tiles + t + 32];
                 int entry = 0;
                 bool need[2] = {false, false};
                 if (t < n_kt) {
-                    const TileSum ts = p.sums[(int64_t)b * p.max_k_tiles + t];
+                    const TileSum ts = kQC ? p.sums[(int64_t)b * p.max_k_tiles + t] : cur;
                     const int k0 = ts.pos_min, k1 = ts.pos_max;  // S_aug positions of the keys
                     const bool kb = ts.flags & 1, kn = ts.flags & 2, ko = ts.flags & 4;
                     entry = (t << 6) | ((kn ? ((kb || ko) ? 2 : 1) : 0) << 4);
@@ -820,7 +899,12 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                            (tile1 ? __popc(__ballot_sync(0xffffffffu, keep && !need[1])) : 0);
                 const unsigned b0 = __ballot_sync(0xffffffffu, need[0]);
                 const unsigned b1 = __ballot_sync(0xffffffffu, need[1]);
-                if (keep) lst[n_list + __popc(bal & ((1u << lane) - 1u))] = entry;
+                const int at = n_list + __popc(bal & ((1u << lane) - 1u));
+                if (kSplit) {  // every S-th listed tile is this block's
+                    if (keep && at % n_split == rank) lst[at / n_split] = entry;
+                } else if (keep) {
+                    lst[at] = entry;
+                }
                 // list index of the last entry each query tile visits
                 if (b0) last0 = n_list + __popc(bal & ((2u << (31 - __clz(b0))) - 1u)) - 1;
                 if (b1) last1 = n_list + __popc(bal & ((2u << (31 - __clz(b1))) - 1u)) - 1;
@@ -828,7 +912,8 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
             }
             // both query tiles visit every listed key tile (masked where they see
             // none of it) unless skipping drops more than a tenth of the products
-            const bool dense = skipped * 10 <= (tile1 ? 2 : 1) * n_list;
+            const bool dense = kSplit || skipped * 10 <= (tile1 ? 2 : 1) * n_list;
+            if (kSplit) n_list = (n_list - rank + n_split - 1) / n_split;
             if (lane == 0) {
                 ui->flags = dense ? 2 : 0;
                 ui->layer = layer;
@@ -858,15 +943,13 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         }
     } else if (warp == 0) {
         // ------------------------------------------------------------ producer
-        if (lane == 0) {
+        if (kQC && lane == 0) {
             tma_prefetch_desc(&tmQ);
             tma_prefetch_desc(&tmK);
             tma_prefetch_desc(&tmV);
-            if (p.key_direct != nullptr) {
-                tma_prefetch_desc(&tmK0);
-                tma_prefetch_desc(&tmV0);
-            }
-            if (p.qchunks != nullptr) tma_prefetch_desc(&tmQ32);
+            tma_prefetch_desc(&tmK0);
+            tma_prefetch_desc(&tmV0);
+            tma_prefetch_desc(&tmQ32);
         }
         int g = 0;  // K/V tiles issued over all units (ring position)
         bool ok = true;
@@ -879,9 +962,12 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
             const int kkstart = ui->kkstart, kklen = ui->kklen;
             const bool udense = ui->flags & 2;  // both query tiles visit every listed tile
             const int32_t *lst = lists + slot * kMaxKTiles;
+            // (the scheduler copied the first unit's Q, whatever its list)
+            const bool q_done = !kQC && k == 0;
+            if (q_done) issued_q = 1;
             if (n_list > 0) {
                 // Q: its buffer is free once the previous unit's last S products are done
-                if (issued_q > 0 &&
+                if (!q_done && issued_q > 0 &&
                     !mbar_wait(q_empty, (issued_q - 1) & 1, p.status, abort_flag))
                     break;
                 if (kQC && lane == 0) {
@@ -927,7 +1013,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                                             q0 + (w & 0xffffff), layer);
                         }
                     }
-                } else if (!kQC && lane == 0) {
+                } else if (!kQC && !q_done && lane == 0) {
                     mbar_arrive_expect_tx(q_full, nq * C::kQBytes);
                     for (int qi = 0; qi < nq; ++qi)
                         tma_load_5d(Qs + qi * C::kQBytes, &tmQ, q_full, 0,
@@ -935,7 +1021,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                                     ui->qstart + ui->qt * urows + qi * (kPair ? 0 : ui->qstepu), 0,
                                     layer);
                 }
-                ++issued_q;
+                if (!q_done) ++issued_q;
                 const int kvh = ui->h0 / p.G;
                 // The key tile's column masks (built once per key tile by the summary
                 // kernel; 8 bytes per lane), where a query tile is cut or the Nexus
@@ -1123,6 +1209,12 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                 const int n_list = ui->n_list, nq = ui->nq;
                 const int last[2] = {ui->last[0], ui->last[1]};
                 const int32_t *lst = lists + slot * kMaxKTiles;
+                if (!kQC && k == 0 && n_list == 0) {
+                    // the first unit's Q is copied even where it has no key tile
+                    ok = mbar_wait(q_full, 0, p.status, abort_flag);
+                    nqu = 1;
+                    tc_commit(q_empty);
+                }
                 if (n_list > 0) {
                     ok = mbar_wait(q_full, nqu & 1, p.status, abort_flag);
                     ++nqu;
@@ -1541,7 +1633,30 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                 const int64_t qrow = (int64_t)ui->qstart + qidx;
                 uint16_t *orow = p.O + layer * p.o_ls + (qrow * p.Hq + h) * D;
                 const int64_t sidx = ((int64_t)layer * p.total_q_rows + qrow) * p.Hq + h;
-                if (last >= 0) {
+                if constexpr (kSplit) {
+                    // the row's part of this block, for the merge below; the buffers it
+                    // goes to are free once both query tiles' last products are done
+                    if (last >= 0) {
+                        if (!mbar_wait(&o_done[0], 0, p.status, abort_flag)) break;
+                        if (ui->nq == 2 && !mbar_wait(&o_done[1], 0, p.status, abort_flag)) break;
+                        tc_fence_after();
+                    }
+                    split_ml[qi * kBM + r] = make_float4(m_used, l, l_lse, ln);
+                    if (last >= 0) {
+#pragma unroll
+                        for (int c = 0; c < D / 32; ++c) {
+                            uint32_t o[32];
+                            tmem_ld32(tO + c * 32, o);
+                            tmem_ld_wait();
+                            reg_fence32(o);
+#pragma unroll
+                            for (int u = 0; u < 8; ++u)
+                                split_o[(qi * (D / 4) + c * 8 + u) * kBM + r] = make_float4(
+                                    __uint_as_float(o[4 * u]), __uint_as_float(o[4 * u + 1]),
+                                    __uint_as_float(o[4 * u + 2]), __uint_as_float(o[4 * u + 3]));
+                        }
+                    }
+                } else if (last >= 0) {
                     // ------------------------------------------------ epilogue
                     if (!mbar_wait(&o_done[qi], (ph >> 3) & 1, p.status, abort_flag)) break;
                     ph ^= 8u;
@@ -1601,6 +1716,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     // After an abort no thread waits any more; let the copies the producer
     // issued land before the block's shared memory goes away.
     if (*abort_flag && warp == 0 && lane == 0) {
+        if (!kQC && misc[3]) issued_q = max(issued_q, 1);
         if (issued_q > 0) mbar_drain(q_full, (issued_q - 1) & 1);
         for (int u = max(0, issued_kv - 2); u < issued_kv; ++u)
             mbar_drain(&kv_full[u & 1], (u >> 1) & 1);
@@ -1610,6 +1726,102 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     }
     __syncthreads();
     if (warp == 1) tmem_dealloc(tmem, 512);
+    if constexpr (kSplit) {
+        // Merge: every block's part read from its shared memory, one warp per 32 rows
+        // (lane = row) and 16 columns; item i is block i % S's.  Two blocks' parts are
+        // loaded at a time: a distributed shared-memory load takes about a microsecond.
+        cluster_sync_all();
+        const UnitInfo *ui = units;
+        constexpr int kCols = 16, kItems = D / kCols;
+        const int n_items = *abort_flag || (ui->flags & 1) ? 0 : ui->nq * (kBM / 32) * kItems;
+        for (int i = rank + warp * n_split; i < n_items; i += n_split * (kPfThreads / 32)) {
+            const int c = i % kItems, row = (i / kItems) * 32 + lane;
+            const int qi = row / kBM, r = row % kBM;
+            constexpr int kMost = 8;
+            float f[kMost];
+            float M = -INFINITY, L = 0.f, Ll = 0.f, Ln = 0.f;
+            float4 ml[kMost];
+#pragma unroll
+            for (int q = 0; q < kMost; ++q)
+                if (q < n_split) ml[q] = ld_cluster_f4(smem_in_rank(split_ml + row, q));
+            float4 a[kCols / 4];
+#pragma unroll
+            for (int u = 0; u < kCols / 4; ++u) a[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+            const float4 *mine = split_o + (qi * (D / 4) + c * (kCols / 4)) * kBM + r;
+            float4 o[2][kCols / 4];
+            auto fetch = [&](int q, float4 (&v)[kCols / 4]) {
+                const uint32_t at = smem_in_rank(mine, q);
+#pragma unroll
+                for (int u = 0; u < kCols / 4; ++u) v[u] = ld_cluster_f4(at + u * kBM * 16);
+            };
+            fetch(0, o[0]);
+            fetch(1, o[1]);
+#pragma unroll
+            for (int q = 0; q < kMost; ++q)
+                if (q < n_split) M = fmaxf(M, ml[q].x);
+#pragma unroll
+            for (int q = 0; q < kMost; ++q) {
+                // (a block that saw no key of the row left its O as it was: not added)
+                f[q] = q < n_split && ml[q].x != -INFINITY ? ex2(ml[q].x - M) : 0.f;
+                if (f[q] != 0.f) {
+                    L += f[q] * ml[q].y;
+                    Ll += f[q] * ml[q].z;
+                    Ln += f[q] * ml[q].w;
+                }
+            }
+            auto add = [&](int q, const float4 (&v)[kCols / 4]) {
+                if (f[q] == 0.f) return;
+#pragma unroll
+                for (int u = 0; u < kCols / 4; ++u) {
+                    a[u].x += f[q] * v[u].x;
+                    a[u].y += f[q] * v[u].y;
+                    a[u].z += f[q] * v[u].z;
+                    a[u].w += f[q] * v[u].w;
+                }
+            };
+#pragma unroll
+            for (int q = 0; q < kMost; q += 2) {
+                if (q >= n_split) break;
+                float4 n[2][kCols / 4];
+#pragma unroll
+                for (int x = 0; x < 2; ++x)
+                    if (q + 2 + x < n_split) fetch(q + 2 + x, n[x]);
+                add(q, o[0]);
+                if (q + 1 < n_split) add(q + 1, o[1]);
+#pragma unroll
+                for (int x = 0; x < 2; ++x)
+#pragma unroll
+                    for (int u = 0; u < kCols / 4; ++u) o[x][u] = n[x][u];
+            }
+            const int qr = r >> pl2, hoff = r & ((1 << pl2) - 1);
+            const int h = ui->h0 + qi * (kPair ? 1 : ui->pairu) + hoff;
+            const int qidx = ui->qt * urows + qi * (kPair ? 0 : ui->qstepu) + qr;
+            if (ui->pbase + qi * (kPair ? 0 : ui->qstepu) + qr > ui->klen - 1 || qidx >= ui->qlen)
+                continue;
+            const float inv = L > 0.f ? 1.f / L : 0.f;
+            const int64_t qrow = (int64_t)ui->qstart + qidx;
+            uint16_t *orow = p.O + ui->layer * p.o_ls + (qrow * p.Hq + h) * D + c * kCols;
+            uint32_t w[8];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                w[2 * u] = pack_bf16x2(a[u].x * inv, a[u].y * inv);
+                w[2 * u + 1] = pack_bf16x2(a[u].z * inv, a[u].w * inv);
+            }
+            if (p.o_v8) {
+                st_global_v8(orow, w);
+            } else {
+                reinterpret_cast<uint4 *>(orow)[0] = make_uint4(w[0], w[1], w[2], w[3]);
+                reinterpret_cast<uint4 *>(orow)[1] = make_uint4(w[4], w[5], w[6], w[7]);
+            }
+            if (c == 0) {
+                const int64_t sidx = ((int64_t)ui->layer * p.total_q_rows + qrow) * p.Hq + h;
+                if (kLse && p.lse != nullptr)
+                    p.lse[sidx] = Ll > 0.f ? (M + __log2f(Ll)) * kLn2f : -INFINITY;
+                if (kMass && p.nexus_mass != nullptr) p.nexus_mass[sidx] = Ln * inv;
+            }
+        }
+        cluster_sync_all();  // no block leaves while another reads its part
+    }
 }
 
 // ---------------------------------------------------------------- key order
@@ -1947,28 +2159,82 @@ kv_permute_kernel(const uint8_t *__restrict__ K, const uint8_t *__restrict__ V,
     }
 }
 
+// Blocks per unit for a call of few units (at most half as many as SMs; with more, a
+// cluster would only move units to a second wave): the most with which all units' clusters are
+// resident at once (one block per SM; clusters do not span the GPU's SM groups, so
+// fewer fit than SMs / size), leaving at least two key tiles to a block.
+template <typename K>
+int split_of(K kern, size_t smem, long long n_units, int max_k_tiles, int head_dim) {
+    // clusters of each size that fit, per device and head_dim (0: not asked yet)
+    static std::atomic<int> most[2][64][9];
+    int dev = 0;
+    if (n_units * 2 > device_sm_count() || cudaGetDevice(&dev) != cudaSuccess) return 1;
+    for (int s = 8; s > 1; --s) {
+        if (s * 2 > max_k_tiles || s * n_units > device_sm_count()) continue;
+        std::atomic<int> *cell = dev < 64 ? &most[head_dim == 128][dev][s] : nullptr;
+        int fit = cell ? cell->load(std::memory_order_relaxed) : 0;
+        if (fit == 0) {
+            cudaLaunchAttribute at{};
+            at.id = cudaLaunchAttributeClusterDimension;
+            at.val.clusterDim.x = s;
+            at.val.clusterDim.y = at.val.clusterDim.z = 1;
+            cudaLaunchConfig_t cfg{};
+            cfg.gridDim = dim3(s);
+            cfg.blockDim = dim3(kPfThreads);
+            cfg.dynamicSmemBytes = smem;
+            cfg.attrs = &at;
+            cfg.numAttrs = 1;
+            if (cudaOccupancyMaxActiveClusters(&fit, kern, &cfg) != cudaSuccess) {
+                (void)cudaGetLastError();
+                fit = 0;
+            }
+            if (cell) cell->store(fit > 0 ? fit : -1, std::memory_order_relaxed);
+        }
+        if (fit >= n_units) return s;
+    }
+    return 1;
+}
+
 template <int D>
 cudaError_t launch_prefill(const CUtensorMap &tq, const CUtensorMap &tk, const CUtensorMap &tv,
                            const CUtensorMap &tk0, const CUtensorMap &tv0, const CUtensorMap &tq32,
-                           const PfParams &p, bool solo, int grid, cudaStream_t s) {
+                           PfParams p, bool solo, int grid, cudaStream_t s) {
     constexpr size_t smem = PfCfg<D>::kSmem;
     static_assert(smem <= 232448, "prefill shared memory");
     const int out = (p.lse != nullptr ? 1 : 0) | (p.nexus_mass != nullptr ? 2 : 0);
     // instances: chunked query order (paired or not), single-tile units, or the
-    // given order (paired or not)
+    // given order (paired or not); each but the first also with its units split
+    // (with no optional output, or able to write both)
     using K = void (*)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap,
                        CUtensorMap, PfParams);
     auto pick = [&](auto qc, auto solo_t, auto pair_t) -> K {
         constexpr bool a = decltype(qc)::value, b = decltype(solo_t)::value,
                        c = decltype(pair_t)::value;
-        return out == 0   ? (K)prefill_kernel<D, 0, a, b, c>
-               : out == 1 ? (K)prefill_kernel<D, 1, a, b, c>
-               : out == 2 ? (K)prefill_kernel<D, 2, a, b, c>
-                          : (K)prefill_kernel<D, 3, a, b, c>;
+        return out == 0   ? (K)prefill_kernel<D, 0, a, b, c, false>
+               : out == 1 ? (K)prefill_kernel<D, 1, a, b, c, false>
+               : out == 2 ? (K)prefill_kernel<D, 2, a, b, c, false>
+                          : (K)prefill_kernel<D, 3, a, b, c, false>;
+    };
+    auto pick_split = [&](auto solo_t, auto pair_t) -> K {
+        constexpr bool b = decltype(solo_t)::value, c = decltype(pair_t)::value;
+        return out == 0 ? (K)prefill_kernel<D, 0, false, b, c, true>
+                        : (K)prefill_kernel<D, 3, false, b, c, true>;
     };
     using T = std::true_type;
     using F = std::false_type;
     const bool paired = p.pair != 0;
+    if (p.qchunks == nullptr) {
+        K kern = solo     ? pick_split(T{}, F{})
+                 : paired ? pick_split(F{}, T{})
+                          : pick_split(F{}, F{});
+        cudaError_t e =
+            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        p.n_split = split_of(kern, smem, p.n_units, p.max_k_tiles, D);
+        if (p.n_split > 1)
+            return launch_pdl(kern, dim3(p.n_units * p.n_split), kPfThreads, smem, s, p.n_split, tq,
+                              tk, tv, tk0, tv0, tq32, p);
+    }
     K kern = p.qchunks != nullptr ? (paired ? pick(T{}, F{}, T{}) : pick(T{}, F{}, F{}))
              : solo               ? pick(F{}, T{}, F{})
              : paired             ? pick(F{}, F{}, T{})
@@ -1976,8 +2242,7 @@ cudaError_t launch_prefill(const CUtensorMap &tq, const CUtensorMap &tk, const C
     cudaError_t e =
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kern<<<grid, kPfThreads, smem, s>>>(tq, tk, tv, tk0, tv0, tq32, p);
-    return cudaGetLastError();
+    return launch_pdl(kern, dim3(grid), kPfThreads, smem, s, 1, tq, tk, tv, tk0, tv0, tq32, p);
 }
 
 // Chunk words per sequence of the retained-first query order: room for
@@ -2226,18 +2491,19 @@ extern "C" sonic_status_t sonic_attn_prefill(const uint16_t *Q, const uint16_t *
         query_order_kernel<<<a->batch, kQOrderThreads, 0, stream>>>(
             role, seg_id, a->k_start, a->k_len, a->q_len, a->max_k_len, a->total_k_rows,
             p.qchunks_per_seq, reinterpret_cast<int32_t *>(wsb + ws.qchunks));
-    tile_summary_kernel<<<dim3(p.max_k_tiles, a->batch), 128, 0, stream>>>(
-        p.key_role, p.key_seg, p.key_pos, p.key_start, p.key_len,
-        reinterpret_cast<TileSum *>(wsb + ws.sums), reinterpret_cast<TileMasks *>(wsb + ws.masks),
-        p.max_k_tiles,
-        reorder ? (int64_t)ws.rows : (int64_t)a->total_k_rows, a->status, p.counter);
     // one persistent block per SM (fewer when there are fewer units)
     const int grid = (int)std::min<long long>(device_sm_count(), n_units);
+    cudaError_t e = launch_pdl(
+        tile_summary_kernel, dim3(p.max_k_tiles, a->batch), 128, 0, stream, 1, p.key_role, p.key_seg,
+        p.key_pos, p.key_start, p.key_len, reinterpret_cast<TileSum *>(wsb + ws.sums),
+        reinterpret_cast<TileMasks *>(wsb + ws.masks), p.max_k_tiles,
+        reorder ? (int64_t)ws.rows : (int64_t)a->total_k_rows, a->status, p.counter,
+        qchunked ? 0 : grid);
+    if (e != cudaSuccess) return SONIC_ERR_CUDA;
     // every unit holds one query tile: packed heads with every query block within
     // one tile (R rows), so the second tile's TMEM block and Q buffer are free
     const bool solo = !qchunked && pack_log2 > 0 && a->max_q_len <= R;
-    cudaError_t e = (D == 128)
-                        ? launch_prefill<128>(tq, tk, tv, tk0, tv0, tq32, p, solo, grid, stream)
+    e = (D == 128)      ? launch_prefill<128>(tq, tk, tv, tk0, tv0, tq32, p, solo, grid, stream)
                         : launch_prefill<64>(tq, tk, tv, tk0, tv0, tq32, p, solo, grid, stream);
     return e == cudaSuccess ? SONIC_OK : SONIC_ERR_CUDA;
 }

@@ -114,3 +114,32 @@ def test_compact_single_launch_scan(n_seqs, rows, total):
     V = inputs.randn((1, batch.total, 1, 8), seed=rows + 1, device=H.dev())
     reserve = rng.integers(0, 5, batch.B)
     _check_compact(batch, K, V, _compact(batch, K, V, reserve=reserve), reserve=reserve)
+
+
+@pytest.mark.parametrize("mode", [sonic.NEXUS_FULL, sonic.NEXUS_CAUSAL_SEGMENTS])
+@pytest.mark.parametrize("hq,hkv,D", [(8, 2, 128), (6, 2, 128), (7, 1, 64), (4, 1, 64)])
+@pytest.mark.parametrize("q", [1, 30, 65, 128, 129, 257, 400])
+def test_prefill_split_units(q, hq, hkv, D, mode):
+    """One or two sequences of few query rows over 5 to 20 key tiles: paired, unpaired and
+    packed units shared by clusters of 2 to 8 blocks, among them blocks without a key
+    tile (a short sequence beside a long one), rows that see keys of some blocks only,
+    with and without the optional outputs."""
+    batch = inputs.Batch([inputs.Dialogue(100, [(130, 20), (260, 0), (0, 33), (400, 60)], q + 900),
+                          inputs.Dialogue(0, [(5, 3), (60, 9)], q)])
+    rows = np.unique(np.r_[0, q // 2, q - 1])
+    for q_len in ([q, q], [min(q + 600, 1000), 0]):
+        res = H.run_prefill(batch, hq, hkv, D, q_len=q_len, seed=q + hq, nexus_vis=mode,
+                            with_mass=True)
+        plain = H.run_prefill(batch, hq, hkv, D, q_len=q_len, nexus_vis=mode, with_lse=False,
+                              K=res["K"], V=res["V"], Q=res["Q"])
+        assert torch.equal(plain["O"].view(torch.int16), res["O"].view(torch.int16))
+        assert torch.isfinite(res["O"].float()).all()
+        for b in range(2):
+            at = rows[rows < q_len[b]]
+            if not len(at):
+                continue
+            O, lse, got, got_lse = H.oracle_prefill_rows(batch, res, b, at, nexus_vis=mode)
+            H.check_close(got, O, f"seq {b}")
+            np.testing.assert_allclose(got_lse, lse, rtol=0, atol=2e-3)
+            want, mass = H.oracle_mass_rows(batch, res, b, at, nexus_vis=mode)
+            np.testing.assert_allclose(mass, want, rtol=0, atol=2e-3)
