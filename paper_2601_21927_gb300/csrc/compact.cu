@@ -204,22 +204,9 @@ keep_scatter_kernel(const uint8_t *__restrict__ role, const int32_t *__restrict_
     }
 }
 
-// Kept rows among n role bytes at p, this thread's share: thread `lane` of `lanes`
-// (>= 16) takes 16-byte words lane, lane + lanes, ... between the unaligned ends.
+// Kept rows among n role bytes at p, this thread's share (see count_equal).
 __device__ __forceinline__ int count_kept(const uint8_t *p, int n, int lane, int lanes) {
-    const int head = min(n, (int)((16 - (reinterpret_cast<uintptr_t>(p) & 15)) & 15));
-    const int words = (n - head) >> 4, tail = (n - head) & 15;
-    int kept = lane < head && p[lane] != SONIC_ROLE_BODY;
-    kept += lane < tail && p[n - tail + lane] != SONIC_ROLE_BODY;
-    const uint4 *w = reinterpret_cast<const uint4 *>(p + head);
-    constexpr uint32_t kBody4 = 0x01010101u * SONIC_ROLE_BODY;
-#pragma unroll 8
-    for (int i = lane; i < words; i += lanes) {
-        const uint4 v = w[i];
-        kept += 16 - (__popc(__vcmpeq4(v.x, kBody4)) + __popc(__vcmpeq4(v.y, kBody4)) +
-                      __popc(__vcmpeq4(v.z, kBody4)) + __popc(__vcmpeq4(v.w, kBody4))) / 8;
-    }
-    return kept;
+    return (lane == 0 ? n : 0) - count_equal(p, n, SONIC_ROLE_BODY, lane, lanes);
 }
 
 // keep_count, keep_bases and keep_scatter in one launch, for calls of at most

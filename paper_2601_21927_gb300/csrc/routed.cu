@@ -4,9 +4,10 @@
 // buffers of their own, each at the row itself or at a caller-given row (so
 // the K and V of new tokens land straight in their retained-cache rows).
 //
-// At most 192 rows take one kernel, routed_small (see there).  More take four
+// At most 192 rows take one kernel, routed_small (see there).  More take these
 // launches, none of which needs a host round trip:
-//   role_count    per 1024-row chunk: its Nexus rows;
+//   role_count    per 1024-row chunk: its Nexus rows (only above 131,072 rows;
+//                 role_order counts for itself below);
 //   role_order    per chunk: the stable partition [ordinary rows | Nexus rows]
 //                 (perm[g] = source row of grouped row g) and the two group
 //                 sizes;
@@ -34,6 +35,8 @@ constexpr int kGBK = 64;          // reduction step (one 128-byte swizzle row)
 constexpr int kGStages = 6;
 constexpr int kGThreads = 192;    // warp 0 TMA, warp 1 MMA (leader), warps 2-5 epilogue
 constexpr int kMaxParts = 4;
+constexpr int kCountRows = 1 << 17;  // rows up to which role_order counts by itself
+constexpr int kEarlyRows = 1 << 14;  // rows up to which the GEMM looks at the roles itself
 
 // ------------------------------------------------------------- partition
 
@@ -58,25 +61,38 @@ role_count_kernel(const uint8_t *__restrict__ role, int32_t T, int32_t *__restri
 }
 
 // Thread = row.  Ordinary rows keep their order at the front, Nexus rows
-// theirs after all ordinary rows.
+// theirs after all ordinary rows.  counts: Nexus rows per chunk, from role_count; NULL
+// (calls of at most kCountRows rows): every block counts the role bytes itself, 16 per
+// load out of L2, which saves that launch.
 __global__ void __launch_bounds__(kChunkRows)
-role_order_kernel(const uint8_t *__restrict__ role, int32_t T, int32_t n_chunks,
-                  const int32_t *__restrict__ counts, int32_t *__restrict__ perm,
-                  int32_t *__restrict__ groups) {
+role_order_kernel(const uint8_t *role, int32_t T, int32_t n_chunks, const int32_t *counts,
+                  int32_t *perm, int32_t *groups) {
+    pdl_wait();
+    pdl_trigger();
     const int c = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     __shared__ int sh_before, sh_total;
     __shared__ int warp_tot[kChunkRows / 32];
-    if (warp == 0) {
+    if (counts == nullptr) {
+        if (tid == 0) sh_before = sh_total = 0;
+        __syncthreads();
+        const int at = c * kChunkRows;
+        int before = count_equal(role, at, SONIC_ROLE_NEXUS, tid, kChunkRows);
+        int total = before + count_equal(role + at, T - at, SONIC_ROLE_NEXUS, tid, kChunkRows);
+        before = __reduce_add_sync(0xffffffffu, before);
+        total = __reduce_add_sync(0xffffffffu, total);
+        if (lane == 0 && total) {
+            atomicAdd(&sh_before, before);
+            atomicAdd(&sh_total, total);
+        }
+    } else if (warp == 0) {
         int before = 0, total = 0;
         for (int i = lane; i < n_chunks; i += 32) {
             const int v = counts[i];
             total += v;
             if (i < c) before += v;
         }
-        for (int o = 16; o > 0; o >>= 1) {
-            before += __shfl_xor_sync(0xffffffffu, before, o);
-            total += __shfl_xor_sync(0xffffffffu, total, o);
-        }
+        before = __reduce_add_sync(0xffffffffu, before);
+        total = __reduce_add_sync(0xffffffffu, total);
         if (lane == 0) {
             sh_before = before;
             sh_total = total;
@@ -123,9 +139,12 @@ __device__ __forceinline__ bool slab_is_run(const int32_t *perm, int s0, int gro
 // Xg[g] = X[perm[g]] for the rows of slabs that are not runs of X: one warp
 // per row, 16-byte loads.
 __global__ void __launch_bounds__(256)
-row_gather_kernel(const uint8_t *__restrict__ X, int64_t x_row_bytes, int32_t T,
-                  int64_t row_bytes, const int32_t *__restrict__ perm,
-                  const int32_t *__restrict__ groups, uint8_t *__restrict__ Xg) {
+row_gather_kernel(const uint8_t *X, int64_t x_row_bytes, int32_t T, int64_t row_bytes,
+                  const int32_t *perm, const int32_t *groups, uint8_t *Xg) {
+    // (before the wait: role_order has let this kernel start only once everything ahead of
+    // the call was complete, which is all that the GEMM reads before its own wait)
+    pdl_trigger();
+    pdl_wait();
     const int lane = threadIdx.x & 31;
     const int64_t n_warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     const int cpr = (int)(row_bytes >> 4);
@@ -160,6 +179,13 @@ row_gather_kernel(const uint8_t *__restrict__ X, int64_t x_row_bytes, int32_t T,
 // reads 96 B/clk of operands from shared memory while the TMA writes another
 // 96 B/clk into it, more than shared memory delivers; the pair form halves
 // the B traffic per SM.
+// A tile takes ~18 us for d_in = 4096, the tensor pipe's own time; calls of few tiles are
+// bound by their number of waves over the 76 pairs and by what runs before the first
+// product, so the partition kernels are two, chained by dependent launches, and the GEMM
+// of a call of one kind of row starts beside them (4096 -> 6144, GPU time in us: 32.7 ->
+// 28.9 at 512 rows, 73.8 -> 69.5 at 2304; 2,304 rows of both kinds 77.7 -> 73.3).  Tiles
+// 192 or 128 columns wide took the same 18 us each and only added waves (700 rows: 30.2
+// at 256 columns, 46.6 at 192, 45.2 at 128).
 
 struct GemmPart {
     uint16_t *base;
@@ -173,6 +199,7 @@ struct GemmParams {
     const int32_t *groups;  // [2]: ordinary rows, Nexus rows
     const int32_t *perm;
     const int32_t *dst_row;
+    const uint8_t *role;
     GemmPart part[kMaxParts];
     int n_parts;
     int T, d_in, d_out, n_tiles_n;
@@ -186,7 +213,7 @@ struct GemmCfg {
     static constexpr int kOffBar = kGStages * kStageBytes;
     static constexpr int kNumBars = 2 * kGStages + 5;
     static constexpr int kOffMisc = kOffBar + kNumBars * 8;
-    static constexpr size_t kSmem = 1024 + kOffMisc + 16;
+    static constexpr size_t kSmem = 1024 + kOffMisc + 16;  // misc: 4 words
 };
 
 // Tile i of the schedule: its grouped-row start, its valid-row end, its
@@ -292,11 +319,6 @@ routed_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t rank = cluster_rank();
     const int cid = blockIdx.x >> 1, n_clusters = gridDim.x >> 1;
-    // no early return: both CTAs of the pair must reach the cluster barriers
-    const int n0 = p.groups[0], n1 = p.groups[1];
-    const int mt0 = (n0 + kGBM - 1) / kGBM, mt1 = (n1 + kGBM - 1) / kGBM;
-    const int total_m = mt0 + mt1;
-    const int n_tiles = timed_out(p.status) ? 0 : total_m * p.n_tiles_n;
     const int nk = p.d_in / kGBK;
 
     if (tid == 0) {
@@ -316,9 +338,37 @@ routed_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
         tmem_alloc_pair(reinterpret_cast<uint32_t *>(&misc[0]), 512);
         tmem_relinquish_pair();
     }
+    if (tid == 0) {
+        tma_prefetch_desc(&tmA);
+        tma_prefetch_desc(&tmX);
+        tma_prefetch_desc(&tmW);
+        tma_prefetch_desc(&tmWn);
+    }
     tc_fence_before();
     cluster_sync_all();  // both CTAs' barriers and tensor memory are set up
     tc_fence_after();
+    pdl_trigger();
+    // Rows of one kind only (an ordinary turn): grouped row g is row g, so the GEMM needs
+    // nothing of the partition and starts at once, beside those kernels (they let this one
+    // start once everything ahead of the call is complete).  Both CTAs of a pair count the
+    // same bytes.  Otherwise it waits for the partition and the copy.
+    int nx = -1;
+    if (p.T <= kEarlyRows) {
+        if (tid == 0) misc[2] = 0;
+        __syncthreads();
+        const int n = __reduce_add_sync(
+            0xffffffffu, count_equal(p.role, p.T, SONIC_ROLE_NEXUS, tid, kGThreads));
+        if (lane == 0 && n) atomicAdd(&misc[2], n);
+        __syncthreads();
+        nx = misc[2];
+    }
+    const bool plain = nx == 0 || nx == p.T;
+    if (!plain) pdl_wait();
+    // no early return: both CTAs of the pair must reach the cluster barriers
+    const int n0 = plain ? p.T - nx : p.groups[0], n1 = plain ? nx : p.groups[1];
+    const int mt0 = (n0 + kGBM - 1) / kGBM, mt1 = (n1 + kGBM - 1) / kGBM;
+    const int total_m = mt0 + mt1;
+    const int n_tiles = timed_out(p.status) ? 0 : total_m * p.n_tiles_n;
     const uint32_t tmem = static_cast<uint32_t>(misc[0]);
 
     int issued = 0;  // pipeline stages this CTA's producer filled (for the drain)
@@ -328,10 +378,6 @@ routed_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
         // count on the leader's `full` barrier, which the leader arms with
         // the pair's bytes.
         if (lane == 0) {
-            tma_prefetch_desc(&tmA);
-            tma_prefetch_desc(&tmX);
-            tma_prefetch_desc(&tmW);
-            tma_prefetch_desc(&tmWn);
             int it = 0;
             bool ok = true;
             for (int i = cid; ok && i < n_tiles; i += n_clusters) {
@@ -340,9 +386,9 @@ routed_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
                 // this CTA's 128 rows of A: straight from X when they are one run
                 // of X's rows, else from the grouped copy
                 const int s0 = w.row0 + (int)rank * kHalfM;
-                const bool run = s0 < w.row_end && slab_is_run(p.perm, s0, w.row_end);
+                const bool run = s0 < w.row_end && (plain || slab_is_run(p.perm, s0, w.row_end));
                 const CUtensorMap *ta = run ? &tmX : &tmA;
-                const int arow = run ? p.perm[s0] : s0;
+                const int arow = run && !plain ? p.perm[s0] : s0;
                 for (int kb = 0; kb < nk; ++kb, ++it) {
                     const int s = it % kGStages;
                     if (it >= kGStages &&
@@ -407,7 +453,7 @@ routed_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
             const GemmTile w = gemm_tile(i, n0, n1, mt0, total_m);
             const int g = w.row0 + (int)rank * kHalfM + r;
             const bool valid = g < w.row_end;
-            const int t = valid ? p.perm[g] : 0;
+            const int t = !valid ? 0 : plain ? g : p.perm[g];
             const int dst = (valid && p.dst_row != nullptr) ? p.dst_row[t] : t;
             if (!mbar_wait(&acc_full[b], (j >> 1) & 1, p.status, abort_flag)) break;
             tc_fence_after();
@@ -464,6 +510,7 @@ routed_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
     }
     __syncthreads();
     cluster_sync_all();  // no CTA leaves while its pair may still touch its memory
+    pdl_wait();          // (nor before the kernels ahead of it, whose workspace the next call reuses)
     tc_fence_after();
     if (warp == 1) tmem_dealloc_pair(tmem, 512);
 }
@@ -512,8 +559,7 @@ constexpr int kSmallRows = 192;
 template <int NT>
 __global__ void __launch_bounds__(kGThreads, 1)
 routed_small_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW,
-                    const __grid_constant__ CUtensorMap tmWn, const uint8_t *role,
-                    const GemmParams p, int n_split) {
+                    const __grid_constant__ CUtensorMap tmWn, const GemmParams p, int n_split) {
     using C = SmallCfg<NT>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>(
@@ -553,7 +599,7 @@ routed_small_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_consta
         for (int w = 0; w < (NT + 31) / 32; ++w) {
             const int t = w * 32 + lane;
             const bool in = t < p.T;
-            const bool nx = in && role[t] == SONIC_ROLE_NEXUS;
+            const bool nx = in && p.role[t] == SONIC_ROLE_NEXUS;
             const uint32_t b = __ballot_sync(0xffffffffu, nx);
             if (__any_sync(0xffffffffu, in && !nx)) kinds |= 1;
             if (b) kinds |= 2;
@@ -723,8 +769,7 @@ int small_split(int tiles, int nk) {
 
 template <int NT>
 cudaError_t launch_small(const uint16_t *X, const CUtensorMap &tW, const CUtensorMap &tWn,
-                         const uint8_t *role, const GemmParams &p, int64_t x_row_stride,
-                         cudaStream_t stream) {
+                         const GemmParams &p, int64_t x_row_stride, cudaStream_t stream) {
     const uint64_t dims[4] = {(uint64_t)p.d_in, (uint64_t)p.T, 1, 1};
     const uint64_t str[3] = {(uint64_t)x_row_stride * 2, (uint64_t)x_row_stride * 2 * p.T,
                              (uint64_t)x_row_stride * 2 * p.T};
@@ -739,7 +784,7 @@ cudaError_t launch_small(const uint16_t *X, const CUtensorMap &tW, const CUtenso
     const int tiles = (p.d_out + kHalfN - 1) / kHalfN;
     const int split = small_split<NT>(tiles, p.d_in / kGBK);
     return launch_pdl(routed_small_kernel<NT>, dim3(tiles * split), kGThreads, smem, stream, split,
-                      tX, tW, tWn, role, p, split);
+                      tX, tW, tWn, p, split);
 }
 
 struct RlWorkspace {
@@ -808,66 +853,74 @@ extern "C" sonic_status_t sonic_routed_linear(const uint16_t *X, const uint16_t 
     const int T = a->n_rows;
     const int chunks = (T + kChunkRows - 1) / kChunkRows;
 
-    // tensor maps: grouped rows of X, and the two weight matrices
-    const uint64_t adims[4] = {(uint64_t)a->d_in, (uint64_t)T, 1, 1};
-    const uint64_t astr[3] = {(uint64_t)a->d_in * 2, (uint64_t)a->d_in * 2 * T,
-                              (uint64_t)a->d_in * 2 * T};
-    // boxes: one CTA's share of a stage (128 rows of A, 128 weight rows)
-    const uint32_t abox[4] = {kGBK, kHalfM, 1, 1};
-    const uint64_t wdims[4] = {(uint64_t)a->d_in, (uint64_t)a->d_out, 1, 1};
-    const uint64_t wstr[3] = {(uint64_t)a->d_in * 2, (uint64_t)a->d_in * 2 * a->d_out,
-                              (uint64_t)a->d_in * 2 * a->d_out};
-    const uint32_t wbox[4] = {kGBK, kHalfN, 1, 1};
-    static_assert(kGBK * kHalfM * 2 == GemmCfg::kABytes && kGBK * kHalfN * 2 == GemmCfg::kBBytes,
-                  "TMA boxes must fill exactly one stage slot");
-    // X itself, for slabs of grouped rows that are runs of X's rows
-    const uint64_t xdims[4] = {(uint64_t)a->d_in, (uint64_t)T, 1, 1};
-    const uint64_t xstr[3] = {(uint64_t)a->x_row_stride * 2, (uint64_t)a->x_row_stride * 2 * T,
-                              (uint64_t)a->x_row_stride * 2 * T};
     p.groups = groups;
     p.perm = perm;
     p.dst_row = a->dst_row;
+    p.role = role;
+    p.n_tiles_n = (a->d_out + kGBN - 1) / kGBN;
     p.n_parts = a->n_parts;
     p.T = T;
     p.d_in = a->d_in;
     p.d_out = a->d_out;
-    p.n_tiles_n = (a->d_out + kGBN - 1) / kGBN;
     p.status = a->status;
-    CUtensorMap tA, tX, tW, tWn;
+    // the two weight matrices: boxes of 128 rows (one CTA's share of a stage)
+    const uint64_t wdims[4] = {(uint64_t)a->d_in, (uint64_t)a->d_out, 1, 1};
+    const uint64_t wstr[3] = {(uint64_t)a->d_in * 2, (uint64_t)a->d_in * 2 * a->d_out,
+                              (uint64_t)a->d_in * 2 * a->d_out};
+    const uint32_t wbox[4] = {kGBK, kHalfN, 1, 1};
+    CUtensorMap tW, tWn;
     if (!make_tmap_bf16_4d(&tW, W, wdims, wstr, wbox) ||
         !make_tmap_bf16_4d(&tWn, W_nexus, wdims, wstr, wbox))
         return SONIC_ERR_INVALID_ARGUMENT;
-    if (T <= kSmallRows) {
-        const cudaError_t e = T <= 16    ? launch_small<16>(X, tW, tWn, role, p, a->x_row_stride, stream)
-                              : T <= 32  ? launch_small<32>(X, tW, tWn, role, p, a->x_row_stride, stream)
-                              : T <= 64  ? launch_small<64>(X, tW, tWn, role, p, a->x_row_stride, stream)
-                              : T <= 128 ? launch_small<128>(X, tW, tWn, role, p, a->x_row_stride, stream)
-                                         : launch_small<192>(X, tW, tWn, role, p, a->x_row_stride, stream);
+    const auto done = [](cudaError_t e) {
         return e == cudaSuccess             ? SONIC_OK
                : e == cudaErrorInvalidValue ? SONIC_ERR_INVALID_ARGUMENT
                                             : SONIC_ERR_CUDA;
+    };
+    if (T <= kSmallRows) {
+        const auto launch = T <= 16    ? launch_small<16>
+                            : T <= 32  ? launch_small<32>
+                            : T <= 64  ? launch_small<64>
+                            : T <= 128 ? launch_small<128>
+                                       : launch_small<192>;
+        return done(launch(X, tW, tWn, p, a->x_row_stride, stream));
     }
-    if (!make_tmap_bf16_4d(&tA, Xg, adims, astr, abox) ||
-        !make_tmap_bf16_4d(&tX, X, xdims, xstr, abox))
+
+    // tensor maps of A (one CTA's 128 rows of a stage): the grouped rows, and X itself for
+    // slabs of grouped rows that are runs of X's rows
+    const uint32_t abox[4] = {kGBK, kHalfM, 1, 1};
+    const uint64_t adims[4] = {(uint64_t)a->d_in, (uint64_t)T, 1, 1};
+    const uint64_t astr[3] = {(uint64_t)a->d_in * 2, (uint64_t)a->d_in * 2 * T,
+                              (uint64_t)a->d_in * 2 * T};
+    const uint64_t xstr[3] = {(uint64_t)a->x_row_stride * 2, (uint64_t)a->x_row_stride * 2 * T,
+                              (uint64_t)a->x_row_stride * 2 * T};
+    CUtensorMap tA, tX;
+    static_assert(kGBK * kHalfM * 2 == GemmCfg::kABytes && kGBK * kHalfN * 2 == GemmCfg::kBBytes,
+                  "TMA boxes must fill exactly one stage slot");
+    if (!make_tmap_bf16_4d(&tA, Xg, adims, astr, abox) || !make_tmap_bf16_4d(&tX, X, adims, xstr, abox))
         return SONIC_ERR_INVALID_ARGUMENT;
 
-    role_count_kernel<<<chunks, 256, 0, stream>>>(role, T, counts);
-    role_order_kernel<<<chunks, kChunkRows, 0, stream>>>(role, T, chunks, counts, perm, groups);
+    if (T > kCountRows) role_count_kernel<<<chunks, 256, 0, stream>>>(role, T, counts);
+    cudaError_t e =
+        launch_pdl(role_order_kernel, dim3(chunks), kChunkRows, 0, stream, 1, role, T, chunks,
+                   T > kCountRows ? (const int32_t *)counts : nullptr, perm, groups);
+    if (e != cudaSuccess) return SONIC_ERR_CUDA;
     const int sms = device_sm_count();
-    const long long gwarps = (long long)sms * 8 * 8;  // 8 blocks of 8 warps per SM at most
+    // 4 blocks of 8 warps per SM at most, which leaves threads for the GEMM's blocks beside them
+    const long long gwarps = (long long)sms * 4 * 8;
     const int gblocks = (int)((T < gwarps ? T : gwarps) + 7) / 8;
-    row_gather_kernel<<<gblocks, 256, 0, stream>>>(
-        reinterpret_cast<const uint8_t *>(X), a->x_row_stride * 2, T, (int64_t)a->d_in * 2, perm,
-        groups, reinterpret_cast<uint8_t *>(Xg));
-
+    e = launch_pdl(row_gather_kernel, dim3(gblocks), 256, 0, stream, 1,
+                   reinterpret_cast<const uint8_t *>(X), a->x_row_stride * 2, T,
+                   (int64_t)a->d_in * 2, perm, groups, reinterpret_cast<uint8_t *>(Xg));
+    if (e != cudaSuccess) return SONIC_ERR_CUDA;
     const long long max_tiles = ((long long)(T + kGBM - 1) / kGBM + 1) * p.n_tiles_n;
     const int pairs = (int)(max_tiles < sms / 2 ? max_tiles : sms / 2);
     const int blocks = 2 * (pairs > 0 ? pairs : 1);
     constexpr size_t smem = GemmCfg::kSmem;
     static_assert(smem <= 232448, "routed GEMM shared memory");
-    cudaError_t e = cudaFuncSetAttribute(routed_gemm_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = cudaFuncSetAttribute(routed_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)smem);
     if (e != cudaSuccess) return SONIC_ERR_CUDA;
-    routed_gemm_kernel<<<blocks, kGThreads, smem, stream>>>(tA, tX, tW, tWn, p);
-    return cudaGetLastError() == cudaSuccess ? SONIC_OK : SONIC_ERR_CUDA;
+    return done(launch_pdl(routed_gemm_kernel, dim3(blocks), kGThreads, smem, stream, 1, tA, tX, tW,
+                           tWn, p));
 }

@@ -39,6 +39,27 @@ __device__ __forceinline__ bool timed_out(const int32_t *status) {
            *reinterpret_cast<const volatile int32_t *>(status) == SONIC_ERR_DEVICE_TIMEOUT;
 }
 
+// ---------------------------------------------------------------- byte counts
+
+// How many of the n bytes at p equal `value`, this thread's share: thread `lane` of
+// `lanes` (>= 16) takes 16-byte words lane, lane + lanes, ... between the unaligned ends.
+__device__ __forceinline__ int count_equal(const uint8_t *p, int n, uint8_t value, int lane,
+                                           int lanes) {
+    const int head = min(n, (int)((16 - (reinterpret_cast<uintptr_t>(p) & 15)) & 15));
+    const int words = (n - head) >> 4, tail = (n - head) & 15;
+    int eq = lane < head && p[lane] == value;
+    eq += lane < tail && p[n - tail + lane] == value;
+    const uint4 *w = reinterpret_cast<const uint4 *>(p + head);
+    const uint32_t v4 = 0x01010101u * value;
+#pragma unroll 8
+    for (int i = lane; i < words; i += lanes) {
+        const uint4 v = w[i];
+        eq += (__popc(__vcmpeq4(v.x, v4)) + __popc(__vcmpeq4(v.y, v4)) +
+               __popc(__vcmpeq4(v.z, v4)) + __popc(__vcmpeq4(v.w, v4))) / 8;
+    }
+    return eq;
+}
+
 // ---------------------------------------------------------------- smem
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {

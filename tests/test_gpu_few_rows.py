@@ -36,6 +36,42 @@ def test_routed_linear_projection_widths(role, T, d_in, cols):
     _check(r)
 
 
+@pytest.mark.parametrize("T", [16384, 16385])
+def test_routed_linear_one_kind_of_row(T):
+    """Both sides of the largest call whose GEMM looks at the roles itself."""
+    r = _run(np.full(T, inputs.ROLE_NEXUS, np.uint8), 64, [32, 32], [False, True], seed=T,
+             cache_rows=T + 77)
+    _check(r, np.r_[0:300, T // 2:T // 2 + 300, T - 300:T])
+
+
+def test_routed_linear_calls_in_a_row_share_a_workspace():
+    """Calls of one kind of row (whose GEMM runs beside the partition kernels) between calls of
+    both kinds, back to back on one workspace."""
+    T, d = 2500, 512
+    W = inputs.randn((256, d), seed=1, device=H.dev())
+    Wn = inputs.randn((256, d), seed=2, device=H.dev())
+    X = [inputs.randn((T, d), seed=3 + k, device=H.dev()) for k in range(6)]
+    roles = [np.full(T, inputs.ROLE_CURR), _roles(T, 1), np.full(T, inputs.ROLE_NEXUS), _roles(T, 2),
+             np.full(T, inputs.ROLE_CURR), _roles(T, 3)]
+    rt = [torch.from_numpy(r.astype(np.uint8)).to(H.dev()) for r in roles]
+    Y = [torch.empty((T, 256), dtype=torch.bfloat16, device=H.dev()) for _ in X]
+    ws = None
+    for _ in range(20):
+        for x, r, y in zip(X, rt, Y):
+            y.zero_()
+            ws = sonic.sonic_routed_linear(x, W, Wn, r, [(y, False)], workspace=ws)
+    torch.cuda.synchronize()
+    for x, r, y in zip(X, rt, Y):
+        one = torch.empty_like(y)
+        sonic.sonic_routed_linear(x, W, Wn, r, [(one, False)])
+        torch.cuda.synchronize()
+        assert torch.equal(one.view(torch.int16), y.view(torch.int16))
+        want = torch.where((r == inputs.ROLE_NEXUS)[:, None], x.float() @ Wn.float().T,
+                           x.float() @ W.float().T)
+        # fp32 sums of 512 products of N(0, 1) values (rms 23), rounded to bf16
+        assert ((y.float() - want).abs() <= 2.0 ** -8 * want.abs() + 0.1).all()
+
+
 @pytest.mark.parametrize("hq,hkv,D,nl", [(32, 8, 128, 1), (28, 4, 128, 3), (4, 2, 64, 2),
                                          (3, 1, 128, 1), (16, 1, 64, 1), (30, 15, 128, 1)])
 @pytest.mark.parametrize("lens", [
