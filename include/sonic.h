@@ -239,7 +239,7 @@ SONIC_API sonic_status_t sonic_attn_prefill(const uint16_t *Q, const uint16_t *K
 /*
  * Workspace bytes for sonic_attn_prefill with these arguments (0 for an empty
  * batch).  AS_GIVEN: 256 bytes for the counter the persistent blocks claim
- * work units from, then 32 + 256 bytes per 128-key tile (its summary and its
+ * work units from and the order they take the sequences in, then 32 + 256 bytes per 128-key tile (its summary and its
  * column masks), batch * ceil(max_k_len / 128) tiles, each part rounded up to
  * 256 bytes.  RETAINED_FIRST counts one more tile per sequence and adds 4
  * bytes per tile, batch * (align128(max_q_len) + 1024) / 8 bytes (the query

@@ -61,6 +61,12 @@ struct TileSum {
     int32_t pos_max;
 };
 
+// Calls of several units per block claim their sequences by length, the longest first:
+// a unit's time grows with its keys (98 key tiles are ~170 us), and claimed late it is
+// what the call ends on.  The order (a byte per sequence) sits behind the unit counter in
+// its 256 bytes of workspace, so up to kSeqOrder sequences; more keep their given order.
+constexpr int kSeqOrder = 252;
+
 // Key rows with role 255 are padding (no key): they count as invalid.
 // `pos` gives each key row's S_aug position (NULL: the row index itself).
 // A k_len outside [0, max_k_len] is refused: the sequence gets no keys.
@@ -102,8 +108,10 @@ struct PfParams {
     int32_t *status;
     const TileSum *sums;
     const TileMasks *masks;  // per key tile, from the summary kernel
+    const uint8_t *seq_order;  // claim order of the sequences; NULL: as given
     int32_t *counter;        // next work unit to claim (set by the summary kernel)
     int n_split;             // kSplit: blocks per unit
+    int n_layers;
     int n_units, qtiles, HG; // units = qtiles x HG x B x n_layers; HG = Hq >> pack_log2
     int max_k_tiles, max_k_len;
     int B, Hq, G;
@@ -304,13 +312,25 @@ tile_summary_kernel(const uint8_t *role, const int32_t *seg,
                     const int32_t *pos, const int32_t *k_start,
                     const int32_t *k_len, TileSum *out,
                     TileMasks *masks_out, int max_k_tiles, int64_t total_rows,
-                    int32_t *status, int32_t *unit_counter, int first_claim) {
+                    int32_t *status, int32_t *unit_counter, int first_claim, uint8_t *order) {
     pdl_wait();
     pdl_trigger();
     const int t = blockIdx.x, b = blockIdx.y;
     // the attention kernel's blocks start with the units of their own indices and claim
     // the others from there (chunked query order: claim every unit, from 0)
     if (t == 0 && b == 0 && threadIdx.x == 0) *unit_counter = first_claim;
+    // the order sequences are claimed in: most keys first (see kSeqOrder)
+    if (order != nullptr && t == 0 && b == 0) {
+        __shared__ int lens[kSeqOrder];
+        const int B = gridDim.y;
+        for (int i = threadIdx.x; i < B; i += blockDim.x) lens[i] = k_len[i];
+        __syncthreads();
+        for (int i = threadIdx.x; i < B; i += blockDim.x) {
+            int rank = 0;
+            for (int j = 0; j < B; ++j) rank += lens[j] > lens[i] || (lens[j] == lens[i] && j < i);
+            order[rank] = (uint8_t)i;
+        }
+    }
     const int len_in = k_len[b];
     // a sequence outside the arrays (or longer than the tiles) gets empty summaries
     const int len = seq_rows(k_start[b], len_in, max_k_tiles * kBN, total_rows);
@@ -513,12 +533,12 @@ __device__ __forceinline__ void tile_mask_bits(const TileMasks *tmk, const uint8
 // three stages (the unused second Q tile's buffer is the third), V of two.
 // kPair: paired units (an even number of query heads per KV head, heads not
 // packed): a unit is one 128-row query block of heads h0 and h0 + 1.
-// kSplit: calls of few units.  A cluster of S blocks shares one unit (block index / S,
-// no counter), each taking every S-th of its listed key tiles, and the blocks merge
-// their partial rows (log-sum-exp, fp32) through distributed shared memory.  Such a call
-// is bound by its longest unit, a chain of ~3.4k clocks per key tile, while most SMs
-// have none: a turn of 333 rows over 2,189 keys (48 units of 17 tiles, S = 2) went from
-// 38 to 29 us, one over 8.7k keys from 126 to 74, 16 rows over 1,872 keys (8 packed
+// kSplit: calls of at most one unit per SM.  A cluster of S >= 1 blocks has one unit (block
+// index / S, no counter), each taking every S-th of its listed key tiles, and for S > 1 the
+// blocks merge their partial rows (log-sum-exp, fp32) through distributed shared memory.
+// Such a call is bound by its longest unit, a chain of ~3.4k clocks per key tile, while the
+// other SMs have none: a turn of 333 rows over 2,189 keys (48 units of 17 tiles, S = 2) went
+// from 38 to 29 us, one over 8.7k keys from 126 to 74, 16 rows over 1,872 keys (8 packed
 // units, S = 7) from 22 to 16, the merge among it (~3 us at S = 2, ~5 at S = 7).
 template <int D, int kOut, bool kQC, bool kSolo, bool kPair, bool kSplit>
 __global__ void __maxnreg__(168)
@@ -528,6 +548,8 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                const PfParams p) {
     using C = PfCfg<D>;
     constexpr bool kLse = kOut & 1, kMass = kOut & 2;
+    // the block starts on its first unit while the tile summaries are still being written
+    constexpr bool kEarly = kSplit || kSolo;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
@@ -619,26 +641,28 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         tmem_alloc(reinterpret_cast<uint32_t *>(&misc[0]), 512);
         tmem_relinquish();
     }
-    if (kQC) pdl_wait();
+    if (!kEarly) pdl_wait();
     pdl_trigger();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = static_cast<uint32_t>(misc[0]);
-    // The summary kernel before this one lets it start once everything ahead of the call is
-    // complete, so the caller's tensors may be read at once: the scheduler warp starts on the
-    // block's first unit (its own index, no claim) and copies its Q while the summaries
-    // are still being written: a call's first product then starts ~3 us earlier (it came
-    // 8 us after the launch; the tiny dialogue's call took 14.5 us, now 11.6).  Everything else waits for them.  (kQC keeps the plain
-    // order: the same start there made the key-tile loops compile 3-7 % slower.)
-    if (!kQC && warp != kSchedWarp) pdl_wait();
+    // kEarly: the summary kernel before this one lets it start once everything ahead of the
+    // call is complete, so the caller's tensors may be read at once: the scheduler warp finds
+    // the block's unit and copies its Q while the summaries are still being written, and
+    // only then waits for them, as everything else does.  With the unit's own index in
+    // place of a claim a call's first product starts ~3 us earlier (it came 8 us after the
+    // launch; the tiny dialogue's call took 14.5 us, now 11.6;
+    // Nexus generation of 256 units 42.8, now 40.2).  The other kernels wait here: with the
+    // later wait in them the key-tile loops compiled 2-7 % slower.
+    if (kEarly && warp != kSchedWarp) pdl_wait();
     // what the producer issued, for the drain after an abort
     int issued_q = 0, issued_kv = 0, issued_k = 0;
 
     if (warp == kSchedWarp) {
         // ------------------------------------------------------------ scheduler
         bool taken = false;  // the block's first unit is taken
-        bool waited = kQC;   // the kernel before this one is complete
+        bool waited = !kEarly;  // the kernel before this one is complete
         for (int k = 0;; ++k) {
             const int slot = k & 1;
             int end = 0, layer = 0, b = 0, hg = 0, qt = 0, cw = 0;
@@ -651,6 +675,10 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                     if (lane == 0 && !*abort_flag && !timed_out(p.status)) u = atomicAdd(p.counter, 1);
                     u = __shfl_sync(0xffffffffu, u, 0);
                 } else if (!taken) {
+                    if (!waited && !kSplit && p.seq_order != nullptr) {
+                        pdl_wait();  // (the summary kernel writes it)
+                        waited = true;
+                    }
                     u = kSplit ? blockIdx.x / n_split : blockIdx.x;
                     dead = timed_out(p.status);  // (tested below, beside the loads that follow)
                     taken = true;
@@ -672,8 +700,13 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                 int rest = u / p.HG;
                 qt = p.qtiles - 1 - rest % p.qtiles;
                 rest /= p.qtiles;
-                b = rest % p.B;
-                layer = rest / p.B;
+                if (!kQC && !kSplit && p.seq_order != nullptr) {
+                    layer = rest % p.n_layers;
+                    b = p.seq_order[rest / p.n_layers];
+                } else {
+                    b = rest % p.B;
+                    layer = rest / p.B;
+                }
                 klen = p.k_len[b];
                 qlen = p.q_len[b];
                 kstart = p.k_start[b];
@@ -856,16 +889,17 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
             int32_t *lst = lists + slot * kMaxKTiles;
             const int n_kt = (kklen + kBN - 1) / kBN;
             int n_list = 0, last0 = -1, last1 = -1, skipped = 0;
-            TileSum next{};  // loaded a step ahead (kQC: when needed)
-            if (!kQC && lane < n_kt) next = p.sums[(int64_t)b * p.max_k_tiles + lane];
+            // kSplit: loaded a step ahead (in the other kernels that, too, cost the loops 3 %)
+            TileSum next{};
+            if (kSplit && lane < n_kt) next = p.sums[(int64_t)b * p.max_k_tiles + lane];
             for (int c0 = 0; c0 < n_kt; c0 += 32) {
                 const int t = c0 + lane;
                 const TileSum cur = next;
-                if (!kQC && t + 32 < n_kt) next = p.sums[(int64_t)b * p.max_k_tiles + t + 32];
+                if (kSplit && t + 32 < n_kt) next = p.sums[(int64_t)b * p.max_k_tiles + t + 32];
                 int entry = 0;
                 bool need[2] = {false, false};
                 if (t < n_kt) {
-                    const TileSum ts = kQC ? p.sums[(int64_t)b * p.max_k_tiles + t] : cur;
+                    const TileSum ts = kSplit ? cur : p.sums[(int64_t)b * p.max_k_tiles + t];
                     const int k0 = ts.pos_min, k1 = ts.pos_max;  // S_aug positions of the keys
                     const bool kb = ts.flags & 1, kn = ts.flags & 2, ko = ts.flags & 4;
                     entry = (t << 6) | ((kn ? ((kb || ko) ? 2 : 1) : 0) << 4);
@@ -1633,7 +1667,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                 const int64_t qrow = (int64_t)ui->qstart + qidx;
                 uint16_t *orow = p.O + layer * p.o_ls + (qrow * p.Hq + h) * D;
                 const int64_t sidx = ((int64_t)layer * p.total_q_rows + qrow) * p.Hq + h;
-                if constexpr (kSplit) {
+                if (kSplit && n_split > 1) {
                     // the row's part of this block, for the merge below; the buffers it
                     // goes to are free once both query tiles' last products are done
                     if (last >= 0) {
@@ -1693,17 +1727,19 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                         }
                     }
                     if (row_ok) {
-                        if (kLse)
+                        // (kSplit: its instance with outputs serves calls that want one)
+                        if (kLse && (!kSplit || p.lse != nullptr))
                             p.lse[sidx] = l_lse > 0.f ? (m_used + __log2f(l_lse)) * kLn2f : -INFINITY;
-                        if (kMass) p.nexus_mass[sidx] = ln * inv;
+                        if (kMass && (!kSplit || p.nexus_mass != nullptr))
+                            p.nexus_mass[sidx] = ln * inv;
                     }
                 } else if (row_ok) {
                     // no key tile to visit (never for a valid layout): zeros
                     uint4 *dst = reinterpret_cast<uint4 *>(orow);
 #pragma unroll
                     for (int u = 0; u < D / 8; ++u) dst[u] = make_uint4(0, 0, 0, 0);
-                    if (kLse) p.lse[sidx] = -INFINITY;
-                    if (kMass) p.nexus_mass[sidx] = 0.f;
+                    if (kLse && (!kSplit || p.lse != nullptr)) p.lse[sidx] = -INFINITY;
+                    if (kMass && (!kSplit || p.nexus_mass != nullptr)) p.nexus_mass[sidx] = 0.f;
                 }
             }
             __syncwarp();
@@ -1726,7 +1762,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     }
     __syncthreads();
     if (warp == 1) tmem_dealloc(tmem, 512);
-    if constexpr (kSplit) {
+    if (kSplit && n_split > 1) {
         // Merge: every block's part read from its shared memory, one warp per 32 rows
         // (lane = row) and 16 columns; item i is block i % S's.  Two blocks' parts are
         // loaded at a time: a distributed shared-memory load takes about a microsecond.
@@ -2203,8 +2239,8 @@ cudaError_t launch_prefill(const CUtensorMap &tq, const CUtensorMap &tk, const C
     static_assert(smem <= 232448, "prefill shared memory");
     const int out = (p.lse != nullptr ? 1 : 0) | (p.nexus_mass != nullptr ? 2 : 0);
     // instances: chunked query order (paired or not), single-tile units, or the
-    // given order (paired or not); each but the first also with its units split
-    // (with no optional output, or able to write both)
+    // given order (paired or not); each but the first also for calls of at most one unit
+    // per SM (with no optional output, or able to write both)
     using K = void (*)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap,
                        CUtensorMap, PfParams);
     auto pick = [&](auto qc, auto solo_t, auto pair_t) -> K {
@@ -2223,7 +2259,7 @@ cudaError_t launch_prefill(const CUtensorMap &tq, const CUtensorMap &tk, const C
     using T = std::true_type;
     using F = std::false_type;
     const bool paired = p.pair != 0;
-    if (p.qchunks == nullptr) {
+    if (p.qchunks == nullptr && p.n_units <= device_sm_count()) {
         K kern = solo     ? pick_split(T{}, F{})
                  : paired ? pick_split(F{}, T{})
                           : pick_split(F{}, F{});
@@ -2231,8 +2267,7 @@ cudaError_t launch_prefill(const CUtensorMap &tq, const CUtensorMap &tk, const C
             cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         p.n_split = split_of(kern, smem, p.n_units, p.max_k_tiles, D);
-        if (p.n_split > 1)
-            return launch_pdl(kern, dim3(p.n_units * p.n_split), kPfThreads, smem, s, p.n_split, tq,
+        return launch_pdl(kern, dim3(p.n_units * p.n_split), kPfThreads, smem, s, p.n_split, tq,
                               tk, tv, tk0, tv0, tq32, p);
     }
     K kern = p.qchunks != nullptr ? (paired ? pick(T{}, F{}, T{}) : pick(T{}, F{}, F{}))
@@ -2452,6 +2487,7 @@ extern "C" sonic_status_t sonic_attn_prefill(const uint16_t *Q, const uint16_t *
     p.masks = reinterpret_cast<const TileMasks *>(wsb + ws.masks);
     p.counter = reinterpret_cast<int32_t *>(wsb + ws.counter);
     p.n_units = (int)n_units;
+    p.n_layers = a->n_layers;
     p.qtiles = (int)qtiles;
     p.HG = (int)HG;
     p.max_k_tiles = max_k_tiles_of(a);
@@ -2491,18 +2527,26 @@ extern "C" sonic_status_t sonic_attn_prefill(const uint16_t *Q, const uint16_t *
         query_order_kernel<<<a->batch, kQOrderThreads, 0, stream>>>(
             role, seg_id, a->k_start, a->k_len, a->q_len, a->max_k_len, a->total_k_rows,
             p.qchunks_per_seq, reinterpret_cast<int32_t *>(wsb + ws.qchunks));
+    // every unit holds one query tile: packed heads with every query block within
+    // one tile (R rows), so the second tile's TMEM block and Q buffer are free
+    const bool solo = !qchunked && pack_log2 > 0 && a->max_q_len <= R;
     // one persistent block per SM (fewer when there are fewer units)
     const int grid = (int)std::min<long long>(device_sm_count(), n_units);
+    // several units per block: sequences claimed by length (GPU time, given order / by
+    // length: eight resuming sequences of 3-12.6k keys, one layer 736 / 706 us, six ragged
+    // ones of two layers 381 / 351, ten shorter ones 135 / 111; layers innermost, so that the
+    // shortest of all layers come last: layer by layer the six took 380).  Single-tile units
+    // start before the order is written, which is worth more to a few.
+    const bool by_len = !qchunked && a->batch > 1 && a->batch <= kSeqOrder && n_units > (solo ? 4LL * grid : grid);
+    uint8_t *order = by_len ? reinterpret_cast<uint8_t *>(p.counter) + 4 : nullptr;
+    p.seq_order = order;
     cudaError_t e = launch_pdl(
         tile_summary_kernel, dim3(p.max_k_tiles, a->batch), 128, 0, stream, 1, p.key_role, p.key_seg,
         p.key_pos, p.key_start, p.key_len, reinterpret_cast<TileSum *>(wsb + ws.sums),
         reinterpret_cast<TileMasks *>(wsb + ws.masks), p.max_k_tiles,
         reorder ? (int64_t)ws.rows : (int64_t)a->total_k_rows, a->status, p.counter,
-        qchunked ? 0 : grid);
+        qchunked ? 0 : grid, order);
     if (e != cudaSuccess) return SONIC_ERR_CUDA;
-    // every unit holds one query tile: packed heads with every query block within
-    // one tile (R rows), so the second tile's TMEM block and Q buffer are free
-    const bool solo = !qchunked && pack_log2 > 0 && a->max_q_len <= R;
     e = (D == 128)      ? launch_prefill<128>(tq, tk, tv, tk0, tv0, tq32, p, solo, grid, stream)
                         : launch_prefill<64>(tq, tk, tv, tk0, tv0, tq32, p, solo, grid, stream);
     return e == cudaSuccess ? SONIC_OK : SONIC_ERR_CUDA;
