@@ -65,7 +65,13 @@ __device__ __forceinline__ bool seq_refused(const DecParams &p, int raw_len, int
 // keys (layer-major, the sequences' lengths one after another); group g of the
 // `groups` blocks of a KV head takes keys [bound(g), bound(g + 1)).  Cuts lie
 // `per` keys apart, moved to a sequence's end where that is less than kSnap keys
-// away, so no piece is shorter than that unless its sequence is.
+// away, so no piece is shorter than that unless its sequence is.  Claimed chunks of
+// ~1/4 of an SM's work left the SMs with up to a chunk more than others (56 ragged
+// sequences of 28/4 heads: 82 us, 4.4 TB/s; in shares 68, 5.3), and short calls with
+// a counter to clear first (16 x 641 rows: 24.4, now 18.8; 64 long ragged ones, four layers:
+// 758, 7.2 TB/s now in 694).  The explicit split (chunk_len) and batches above kSeqCache
+// sequences, or KV heads that leave over an eighth of the SMs without a group, keep the
+// chunks.
 constexpr int kMinShare = 64;
 constexpr int kSnap = 32;
 
@@ -820,12 +826,16 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
 template <int D>
 __global__ void __launch_bounds__(128)
 decode_combine_kernel(const DecParams p, int n_layers) {
-    pdl_wait();
-    pdl_trigger();
+    // The main kernel lets this one start once everything ahead of the call is complete, so
+    // the lengths are read and the pieces found while it still runs (1.0-1.5 us less behind
+    // every call: 1 x 641 rows 10.8 -> 9.8 us, 16 x 641 19.9 -> 18.8).
     const int64_t unit = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     const int64_t n_units = (int64_t)n_layers * p.B * p.Hq;
-    if (unit >= n_units) return;
+    if (unit >= n_units) {
+        pdl_wait();  // (no block ends before the main kernel: the next call reuses its workspace)
+        return;
+    }
     const int h = (int)(unit % p.Hq);
     const int64_t lb = unit / p.Hq;
     const int b = (int)(lb % p.B), layer = (int)(lb / p.B);
@@ -854,6 +864,8 @@ decode_combine_kernel(const DecParams p, int n_layers) {
         step = (int64_t)p.Hkv * 2 * heads;
         slot1 = slot0 - heads;
     }
+    pdl_wait();
+    pdl_trigger();
     if (n == 1) return;  // written by the split kernel
     uint16_t *op = p.O + layer * p.o_ls + ((int64_t)b * p.Hq + h) * D;
     constexpr int kDpl = D / 32;
