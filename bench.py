@@ -174,7 +174,9 @@ class GpuStep:
         self.outV = self.Vret[:, lay.T_dec:]
         # workspaces (caller-owned; sized once)
         self.ws_c = self.ws_p = self.ws_d = None
-        self.launches_per_step = 4 + 2 + 2
+        # compaction (one scan launch up to 2^19 raw rows, else three, and the copy),
+        # prefill and decode
+        self.launches_per_step = (2 if self.raw_role.numel() <= 1 << 19 else 4) + 2 + 2
 
     def compact(self, stream=None):
         self.ws_c = self.sonic.sonic_compact_kv(

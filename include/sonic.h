@@ -294,7 +294,7 @@ typedef struct {
     int32_t n_heads_kv;          /* Hkv >= 1                                            */
     int32_t head_dim;            /* D: 64 or 128                                        */
     const int32_t *kv_start;     /* device [B]: first retained row of sequence b         */
-    int32_t max_len;             /* host: >= every lens[b]; sizes the split grid        */
+    int32_t max_len;             /* host: >= every lens[b]; sizes the split             */
     int32_t total_kv_rows;       /* rows per layer of K_ret and V_ret                   */
     int64_t q_layer_stride;      /* elements between layers of q                        */
     int64_t kv_layer_stride;     /* elements between layers of K_ret and V_ret          */
@@ -317,21 +317,23 @@ typedef struct {
  * given); for sequence b the retained rows kv_start[b] .. kv_start[b] +
  * lens[b] - 1 of K_ret / V_ret (the new token's own row included) are all
  * visible:  O[l, b, h] = sum_t softmax_t(scale <q[l,b,h], K[t, h/G]>) V[t, h/G].
- * The keys are split into chunks of chunk_len; each (layer, sequence, KV
- * head, chunk) unit produces a partial (max, sum, accumulator) in the
- * workspace, and a second kernel merges them by log-sum-exp (a sequence that
- * fits one chunk is written directly).  One persistent block per SM claims
- * units from a counter in the workspace (zeroed on `stream` before the
- * launch), so the workspace is never empty and concurrent calls need
- * workspaces of their own.  A sequence whose rows fall outside [0, total_kv_rows) is
+ * One persistent block per SM takes an equal share of the keys of one KV head;
+ * a sequence cut between blocks leaves a partial (max, sum, accumulator) of
+ * each piece in the workspace, and a second kernel merges them by log-sum-exp
+ * (a sequence within one share is written directly).  With chunk_len > 0 (or
+ * more than 1024 sequences, or a number of KV heads that suits the SMs badly)
+ * the keys are split into chunks instead, whose (layer, sequence, KV head,
+ * chunk) units the blocks claim from a counter in the workspace (zeroed on
+ * `stream` before the launch).  The workspace is never empty, and concurrent
+ * calls need workspaces of their own.  A sequence whose rows fall outside [0, total_kv_rows) is
  * refused with SONIC_ERR_INVALID_ARGUMENT in *status (its outputs are left
  * undefined).  lens[b] = 0 gives zeros (and
  * lse = -inf).  bf16 in/out, fp32 arithmetic.  nexus_mass (optional, role
  * then required, else SONIC_ERR_INVALID_ARGUMENT) is the decode form of the
  * quantity behind A_nexus (Sec. 4.1, Eq. 9): the share of the new token's
  * attention, per query head, on retained rows t with role[kv_start[b] + t]
- * = SONIC_ROLE_NEXUS (0 when lens[b] = 0); it adds one float per (unit,
- * chunk) to the workspace.
+ * = SONIC_ROLE_NEXUS (0 when lens[b] = 0); it adds one float per partial to
+ * the workspace.
  */
 SONIC_API sonic_status_t sonic_attn_decode(const uint16_t *q, const uint16_t *K_ret,
                                  const uint16_t *V_ret, const int32_t *lens, uint16_t *O,

@@ -5,14 +5,14 @@
 // kept).  Every retained row of a sequence is visible to its new token.
 //
 // Split-K, HBM-bound design:
-//   decode_tc      persistent blocks (one per SM) claim units (key chunk, KV
-//                  head, sequence, layer) from a counter and stream their K/V
-//                  tiles of 128 keys through a TMA ring; both contractions run
+//   decode_tc      persistent blocks (one per SM) take equal shares of the keys
+//                  (or, for an explicit split, claim key chunks from a counter)
+//                  and stream their K/V tiles of 128 keys through a TMA ring; both contractions run
 //                  on the tensor cores with the keys in the M dimension (see
 //                  the kernel's comment); a single-chunk sequence writes O
 //                  directly, otherwise the partial (max, sum, unnormalised
-//                  accumulator) goes to the workspace.  head_dim 64 and 128.
-//   decode_combine log-sum-exp merge of the chunks of each (layer, seq, head).
+//                  accumulator) of each piece goes to the workspace.  head_dim 64 and 128.
+//   decode_combine log-sum-exp merge of the pieces of each (layer, seq, head).
 // K and V are read exactly once from HBM; softmax runs in base 2.
 #include <type_traits>
 
@@ -130,10 +130,11 @@ __device__ __forceinline__ float warp_max(float v) {
 // O rescale.  S^T and P are double buffered so S^T of the next tile overlaps
 // the softmax and P.V of the current one.
 //
-// The kernel is persistent: one block per SM claims units (key chunk, KV
-// head, sequence, layer) from a global counter (so ragged units balance over
-// the SMs) and works through them as one continuous stream of key tiles: the
-// K/V ring and the tensor pipe stay busy across unit boundaries (the next
+// The kernel is persistent: one block per SM takes an equal share of the keys
+// of one KV head (see above; adjacent blocks hold the KV heads of the same rows) or,
+// for an explicit split, claims units (key chunk, KV head, sequence, layer) from a
+// global counter, and works through its units as one continuous stream of key tiles:
+// the K/V ring and the tensor pipe stay busy across unit boundaries (the next
 // unit's q is staged and its first S^T issued while the current unit
 // finishes).  q and the O^T accumulator are double buffered by unit.  Short
 // sequences (a few tiles per unit) would otherwise spend most of a block's
@@ -369,12 +370,12 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
             cur = cut(grp, sl, sb, off);
             end = cut(grp + 1, l1, b1, o1);
         }
-        // Lane 0 finds its units (equal shares) or claims them from the counter, publishes each in the unit
-        // queue and streams its q (one TMA box of 16 heads: rows past the
-        // group's G heads are other heads' q or zeros, whose S^T columns the
-        // softmax never reads) and its K/V tiles.  The claim of unit k + 1 is
-        // sent before unit k's copies are queued; its answer is needed only
-        // after them.
+        // Lane 0 finds its units (equal shares) or claims them from the counter,
+        // publishes each in the unit queue and streams its q (one TMA box of 16
+        // heads: rows past the group's G heads are other heads' q or zeros, whose
+        // S^T columns the softmax never reads) and its K/V tiles.  A claim of unit
+        // k + 1 is sent before unit k's copies are queued; its answer is needed
+        // only after them.
         if (lane == 0) {
             int T = 0;  // K/V tiles issued
             auto next_share = [&](TcUnit &w) -> bool {
@@ -1009,7 +1010,8 @@ Plan make_plan(const sonic_decode_args *a) {
 }
 
 // Persistent launch: one block per SM (the stage ring takes most of shared
-// memory); the blocks claim units from a counter zeroed on the stream first.
+// memory).  In equal shares the blocks know their keys; otherwise they claim
+// units from a counter zeroed on the stream first.
 struct TcMaps {
     CUtensorMap k, v, q, k16, v16;
 };
