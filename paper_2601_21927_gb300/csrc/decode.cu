@@ -751,10 +751,11 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                     if (want_nx) n[g] = n[g] * alpha[g] + (isn ? __bfloat162float(pr) : 0.f);
                     *reinterpret_cast<__nv_bfloat16 *>(pb + g * 128 + ((jj ^ (g & 7)) << 4)) = pr;
                 }
-                if (!valid) {
-                    // rows of a partial tile past the unit's keys (another sequence's,
-                    // junk, or what shared memory held): zero their V, so 0 * garbage
-                    // cannot reach O (their K only makes scores that are masked)
+                if (!valid && (T < kTcStages || r < ((w.nkeys - t * kTcKeys + 15) & ~15))) {
+                    // rows of a partial tile past the unit's keys (another sequence's or
+                    // junk; in a stage's first tile also what shared memory held, later
+                    // an earlier tile's rows): zero their V, so 0 * garbage cannot reach O
+                    // (their K only makes scores that are masked)
                     uint8_t *vrow =
                         smem + (T % kTcStages) * C::kStageBytes + C::kTileBytes + r * 128;
 #pragma unroll
