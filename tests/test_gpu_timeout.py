@@ -103,3 +103,23 @@ def test_decode_wait_timeout_then_normal_call(short_wait_lib):
             Oref, _ = oracle.decode(H.f64(q[layer, b]), H.f64(K[layer, s0:s0 + n]),
                                     H.f64(V[layer, s0:s0 + n]))
             H.check_close(H.f64(O[layer, b]), Oref, f"layer {layer} seq {b}")
+
+
+@pytest.mark.parametrize("case", ["paired", "single_tile", "unpaired"])
+def test_prefill_wait_timeout_with_several_units_per_block(short_wait_lib, case):
+    """The same with enough sequences that the persistent blocks claim several units each (the
+    calls above have at most one unit per SM, which takes instances of its own)."""
+    c = PREFILL_CASES[case]
+    rng = np.random.default_rng(22)
+    n = 160 if c["short"] else 48
+    batch = inputs.Batch([inputs.random_dialogue(rng, max_segments=5, max_body=400,
+                                                 max_nexus=40, max_curr=300) for _ in range(n)])
+    q_len = np.minimum(batch.k_len, 32).astype(np.int32) if c["short"] else None
+    args = dict(hq=c["hq"], hkv=c["hkv"], D=128, seed=4, key_order=c["order"], q_len=q_len)
+    _with(short_wait_lib, lambda: H.run_prefill(batch, expect_status=TIMEOUT, **args))
+    torch.cuda.synchronize()
+    res = H.run_prefill(batch, **args)
+    for b in (0, 17, n - 1):
+        O, lse, got, got_lse = H.oracle_prefill_rows(batch, res, b, np.arange(res["q_len"][b]))
+        H.check_close(got, O, f"seq {b}")
+        np.testing.assert_allclose(got_lse, lse, rtol=0, atol=2e-3)
