@@ -1677,11 +1677,15 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                 const int64_t sidx = ((int64_t)layer * p.total_q_rows + qrow) * p.Hq + h;
                 if (kSplit && n_split > 1) {
                     // the row's part of this block, for the merge below; the buffers it
-                    // goes to are free once both query tiles' last products are done
+                    // goes to are free once both query tiles' last products are done, or,
+                    // in a block without a key tile, once the Q that the scheduler copied
+                    // (which nothing reads) has landed: later it would fall on split_ml
                     if (last >= 0) {
                         if (!mbar_wait(&o_done[0], 0, p.status, abort_flag)) break;
                         if (ui->nq == 2 && !mbar_wait(&o_done[1], 0, p.status, abort_flag)) break;
                         tc_fence_after();
+                    } else if (!mbar_wait(q_full, 0, p.status, abort_flag)) {
+                        break;
                     }
                     split_ml[qi * kBM + r] = make_float4(m_used, l, l_lse, ln);
                     if (last >= 0) {

@@ -179,3 +179,37 @@ def test_prefill_split_units(q, hq, hkv, D, mode):
             np.testing.assert_allclose(got_lse, lse, rtol=0, atol=2e-3)
             want, mass = H.oracle_mass_rows(batch, res, b, at, nexus_vis=mode)
             np.testing.assert_allclose(mass, want, rtol=0, atol=2e-3)
+
+
+@pytest.mark.parametrize("hq,hkv,D,n", [(2, 1, 64, 2048), (2, 1, 128, 1024), (8, 2, 128, 2048),
+                                        (8, 2, 128, 1024), (3, 1, 64, 1500)])
+def test_prefill_split_blocks_without_a_key_tile(hq, hkv, D, n):
+    """Every row of one sequence, layer by layer: the first query blocks list fewer key tiles than
+    their cluster has blocks (a block without one copies its Q for nothing, and its part of the
+    rows goes over that copy).  All rows against a call over so many layers that no unit is split,
+    20 times over with Q out of L2, bit for bit the same each time."""
+    batch = inputs.Batch([inputs.Dialogue(400, [(200, 20), (0, 0), (300, 9)], n - 929)])
+    nl = 12 * 8 // hq + 8
+    res = H.run_prefill(batch, hq, hkv, D, seed=n + hq, n_layers=nl, with_mass=True)
+    role, seg, k_start, k_len = H.meta(batch)
+    flush = torch.empty(1 << 28, dtype=torch.uint8, device=H.dev())
+    first, ws = {}, None
+    for i in range(20):
+        l = i % 2 * (nl - 1)
+        O = torch.full_like(res["O"][:1], float("nan"))
+        lse, mass = torch.full_like(res["lse"][:1], 7.0), torch.full_like(res["mass"][:1], 7.0)
+        status = torch.zeros(1, dtype=torch.int32, device=H.dev())
+        flush.fill_(i)
+        ws = sonic.sonic_attn_prefill(
+            res["Q"][l:l + 1], res["K"][l:l + 1], res["V"][l:l + 1], seg, role, O, k_start=k_start,
+            k_len=k_len, q_start=k_start, q_len=k_len, max_q_len=n, max_k_len=n, lse=lse,
+            nexus_mass=mass, status=status, workspace=ws)
+        torch.cuda.synchronize()
+        assert sonic.read_status(status) == 0
+        got = (O.view(torch.int16), lse, mass)
+        if l not in first:
+            first[l] = got
+            H.check_close(H.f64(O[0]), H.f64(res["O"][l]), f"layer {l}")
+            np.testing.assert_allclose(H.f64(lse[0]), H.f64(res["lse"][l]), rtol=0, atol=2e-3)
+            np.testing.assert_allclose(H.f64(mass[0]), H.f64(res["mass"][l]), rtol=0, atol=2e-3)
+        assert all(torch.equal(a, b) for a, b in zip(first[l], got))
