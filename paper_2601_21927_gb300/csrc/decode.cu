@@ -459,7 +459,7 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                     } else {
                         // a unit's last, partial tile: only its rows, in 16-row boxes
                         // (the rows past them keep older data; the softmax masks
-                        // their scores and zeroes their V rows)
+                        // their scores, and P.V leaves their V rows out)
                         const int nb = (rem + 15) / 16;
                         mbar_arrive_expect_tx(&full[s], nb * 2 * kLoads * (16 * 128));
                         for (int j = 0; j < nb; ++j)
@@ -567,17 +567,30 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                     tc_fence_after();
                     const uint32_t v_addr = base + (T % kTcStages) * C::kStageBytes + C::kTileBytes;
                     const uint32_t pb = p_addr + (T & 1) * C::kPBytes;
+                    auto issue_pv = [&](int hh, int kk) {
+                        const uint64_t a = smem_desc_sw128(
+                            v_addr + hh * (kTcKeys * 128) + kk * (16 * 128), kTcKeys * 128, 1024);
+                        const uint64_t bd = smem_desc_sw128(
+                            pb + (kk >> 2) * (kTcN * 128) + (kk & 3) * 32, 16, 1024);
+                        tc_mma_ss(tO + (k & 1) * kSStride + hh * kTcN, a, bd, idPV,
+                                  (t > 0 || kk > 0) ? 1u : 0u);
+                    };
+                    const int rem = w.nkeys - t * kTcKeys;
+                    if (rem >= kTcKeys) {
 #pragma unroll
-                    for (int hh = 0; hh < (kPair ? 2 : 1); ++hh)
+                        for (int hh = 0; hh < (kPair ? 2 : 1); ++hh)
 #pragma unroll
-                        for (int kk = 0; kk < kTcKeys / 16; ++kk) {
-                            const uint64_t a = smem_desc_sw128(
-                                v_addr + hh * (kTcKeys * 128) + kk * (16 * 128), kTcKeys * 128, 1024);
-                            const uint64_t bd = smem_desc_sw128(
-                                pb + (kk >> 2) * (kTcN * 128) + (kk & 3) * 32, 16, 1024);
-                            tc_mma_ss(tO + (k & 1) * kSStride + hh * kTcN, a, bd, idPV,
-                                      (t > 0 || kk > 0) ? 1u : 0u);
-                        }
+                            for (int kk = 0; kk < kTcKeys / 16; ++kk) issue_pv(hh, kk);
+                    } else {
+                        // a partial tile: only the 16-key steps it has.  V rows behind its
+                        // last copy hold an earlier tile's (another sequence's) rows, and
+                        // 0 * Inf or NaN is NaN.  (Tested in the loop above, the end of the
+                        // tile cost full tiles 0.3-1 % of long calls.)
+#pragma unroll 1
+                        for (int kk = 0; kk * 16 < rem; ++kk)
+#pragma unroll
+                            for (int hh = 0; hh < (kPair ? 2 : 1); ++hh) issue_pv(hh, kk);
+                    }
                     tc_commit(o_done);
                     tc_commit(&empty[T % kTcStages]);
                     if (t == w.ntiles - 1) tc_commit(&o_last[k & 1]);
@@ -751,11 +764,10 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                     if (want_nx) n[g] = n[g] * alpha[g] + (isn ? __bfloat162float(pr) : 0.f);
                     *reinterpret_cast<__nv_bfloat16 *>(pb + g * 128 + ((jj ^ (g & 7)) << 4)) = pr;
                 }
-                if (!valid && (T < kTcStages || r < ((w.nkeys - t * kTcKeys + 15) & ~15))) {
-                    // rows of a partial tile past the unit's keys (another sequence's or
-                    // junk; in a stage's first tile also what shared memory held, later
-                    // an earlier tile's rows): zero their V, so 0 * garbage cannot reach O
-                    // (their K only makes scores that are masked)
+                if (!valid && r < ((w.nkeys - t * kTcKeys + 15) & ~15)) {
+                    // rows a partial tile loaded past the unit's keys (another sequence's, or
+                    // junk): zero their V, so 0 * garbage cannot reach O (their K only makes
+                    // scores that are masked; P.V takes no rows behind these)
                     uint8_t *vrow =
                         smem + (T % kTcStages) * C::kStageBytes + C::kTileBytes + r * 128;
 #pragma unroll

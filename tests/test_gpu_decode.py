@@ -178,3 +178,36 @@ def test_very_long_cache():
     merged), next to a one-row sequence."""
     r = _decode([500_000, 1], 8, 2, 128, n_layers=1, seed=41, pad=3)
     _check(r, [(0, 0), (0, 1)])
+
+
+@pytest.mark.parametrize("chunk_len", [0, 128])
+@pytest.mark.parametrize("hq,hkv,D,nl", [(32, 8, 128, 4), (8, 2, 128, 1), (8, 4, 64, 6), (2, 1, 64, 2)])
+@pytest.mark.parametrize("bad", [float("inf"), float("nan")])
+def test_nonfinite_rows_stay_in_their_sequence(hq, hkv, D, nl, chunk_len, bad):
+    """Infinities or NaN in the K and V of the long sequences, short ones after them in the same
+    blocks (whose last tiles leave rows of the earlier tiles in shared memory): the short ones'
+    outputs do not change by a bit."""
+    lens = np.array([600, 37, 900, 5, 300, 1, 2049, 130] * 4 + [700] * 2, np.int32)
+    starts = np.concatenate([[0], np.cumsum(lens)[:-1]]).astype(np.int32)
+    T = int(lens.sum())
+    K = inputs.randn((nl, T, hkv, D), seed=1, device=H.dev())
+    V = inputs.randn((nl, T, hkv, D), seed=2, device=H.dev())
+    q = inputs.randn((nl, len(lens), hq, D), seed=3, device=H.dev())
+
+    def run():
+        O = torch.full_like(q, float("nan"))
+        lse = torch.empty(q.shape[:3], device=H.dev())
+        sonic.sonic_attn_decode(q, K, V, H.i32(lens), O, kv_start=H.i32(starts),
+                                max_len=int(lens.max()), lse=lse, chunk_len=chunk_len)
+        torch.cuda.synchronize()
+        return O, lse
+
+    O, lse = run()
+    for b in np.flatnonzero(lens >= 600):
+        V[:, starts[b]:starts[b] + lens[b]] = bad
+        K[:, starts[b]:starts[b] + lens[b]] = bad
+    O2, lse2 = run()
+    clean = torch.from_numpy(np.flatnonzero(lens < 600)).to(H.dev())
+    assert torch.isfinite(O[:, clean]).all()
+    assert torch.equal(O[:, clean].view(torch.int16), O2[:, clean].view(torch.int16))
+    assert torch.equal(lse[:, clean], lse2[:, clean])
