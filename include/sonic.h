@@ -304,7 +304,8 @@ typedef struct {
                                     tile of 128 keys                                    */
     float *lse;                  /* device [n_layers][B][Hq] or NULL                    */
     int32_t *status;             /* device int32 or NULL                                */
-    void *workspace;             /* device, sonic_decode_workspace_size() bytes         */
+    void *workspace;             /* device, sonic_decode_workspace_size() bytes, at any
+                                    alignment                                            */
     size_t workspace_bytes;
     const uint8_t *role;         /* device [total_kv_rows] or NULL: role of each retained
                                     row (needed for nexus_mass)                         */

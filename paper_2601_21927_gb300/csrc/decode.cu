@@ -971,12 +971,15 @@ int g_template(int G) {
     return 0;
 }
 
+constexpr size_t kWsAlign = 16;
+
 struct Plan {
     int chunk_len, max_chunks;
     int groups;  // > 0: equal shares
     // partial accumulators, partial (max, sum), partial Nexus sums, unit counter
     size_t ws_acc, ws_ml, ws_nx, ws_cnt;
-    size_t total() const { return ws_acc + ws_ml + ws_nx + ws_cnt; }
+    // (with room to start on a 16-byte boundary of any workspace: the merge loads float4)
+    size_t total() const { return ws_acc + ws_ml + ws_nx + ws_cnt + kWsAlign; }
 };
 
 // head_dim 64 with G <= 8 and an even number of KV heads: units of two KV heads.
@@ -1157,10 +1160,11 @@ extern "C" sonic_status_t sonic_attn_decode(const uint16_t *q, const uint16_t *K
     p.lens = lens;
     p.kv_start = a->kv_start;
     p.lse = a->lse;
-    p.part_acc = static_cast<float *>(a->workspace);
-    p.part_ml = reinterpret_cast<float *>(static_cast<char *>(a->workspace) + pl.ws_acc);
-    p.part_nx =
-        reinterpret_cast<float *>(static_cast<char *>(a->workspace) + pl.ws_acc + pl.ws_ml);
+    char *wsb = reinterpret_cast<char *>(
+        (reinterpret_cast<uintptr_t>(a->workspace) + kWsAlign - 1) & ~(uintptr_t)(kWsAlign - 1));
+    p.part_acc = reinterpret_cast<float *>(wsb);
+    p.part_ml = reinterpret_cast<float *>(wsb + pl.ws_acc);
+    p.part_nx = reinterpret_cast<float *>(wsb + pl.ws_acc + pl.ws_ml);
     p.role = a->role;
     p.nexus_mass = a->nexus_mass;
     p.status = a->status;
@@ -1180,8 +1184,7 @@ extern "C" sonic_status_t sonic_attn_decode(const uint16_t *q, const uint16_t *K
     const float scale = a->softmax_scale > 0.f ? a->softmax_scale : 1.0f / sqrtf((float)D);
     p.scale_log2 = scale * kLog2e;
 
-    int *counter = reinterpret_cast<int *>(static_cast<char *>(a->workspace) + pl.ws_acc +
-                                           pl.ws_ml + pl.ws_nx);
+    int *counter = reinterpret_cast<int *>(wsb + pl.ws_acc + pl.ws_ml + pl.ws_nx);
     const int n_units = (int)(units_x * a->batch * a->n_layers);
     cudaError_t e =
         D == 128 ? dispatch_tc<128, false>(GT, tm, p, (int)units_x, n_units, counter, stream)

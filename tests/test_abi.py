@@ -168,3 +168,13 @@ def test_routed_linear_validation():
     a.parts[0].rows = 10
     assert lib.sonic_routed_linear(16, 16, 16, 16, ctypes.byref(a), None) == 3  # no workspace
     assert lib.sonic_routed_linear_workspace_size(ctypes.byref(a)) == 256 + 256 + 256 + 2560
+
+
+def test_decode_workspace_has_room_for_any_alignment():
+    """The merge loads float4 from the workspace, which may start at any address: 16 bytes more than
+    its parts (here the 256 bytes of the unit counter alone: one chunk holds every sequence)."""
+    lib = sonic.load()
+    d = sonic.sonic_decode_args()
+    d.batch, d.n_layers, d.n_heads_q, d.n_heads_kv, d.head_dim = 2, 1, 8, 2, 128
+    d.max_len, d.total_kv_rows, d.chunk_len = 10, 20, 128
+    assert lib.sonic_decode_workspace_size(ctypes.byref(d)) == 256 + 16

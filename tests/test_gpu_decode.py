@@ -211,3 +211,38 @@ def test_nonfinite_rows_stay_in_their_sequence(hq, hkv, D, nl, chunk_len, bad):
     assert torch.isfinite(O[:, clean]).all()
     assert torch.equal(O[:, clean].view(torch.int16), O2[:, clean].view(torch.int16))
     assert torch.equal(lse[:, clean], lse2[:, clean])
+
+
+@pytest.mark.parametrize("D,hq,chunk_len,with_mass", [(128, 8, 0, True), (128, 28, 256, False),
+                                                      (64, 8, 0, False), (64, 6, 128, True)])
+@pytest.mark.parametrize("offset", [0, 1, 4, 8, 12, 255])
+def test_workspace_at_any_alignment(D, hq, chunk_len, with_mass, offset):
+    """A workspace of just the bytes asked for, `offset` bytes into a larger buffer: the same
+    outputs to the bit, and nothing written around it."""
+    hkv = 4 if hq == 28 else 2
+    lens = np.array([1, 700, 2049, 0, 129], np.int32)
+    starts = np.concatenate([[0], np.cumsum(lens)[:-1]]).astype(np.int32)
+    T = int(lens.sum())
+    K = inputs.randn((2, T, hkv, D), seed=1, device=H.dev())
+    V = inputs.randn((2, T, hkv, D), seed=2, device=H.dev())
+    q = inputs.randn((2, len(lens), hq, D), seed=3, device=H.dev())
+    role = torch.full((T,), inputs.ROLE_NEXUS, dtype=torch.uint8, device=H.dev())
+    role[::3] = inputs.ROLE_CURR
+
+    def run(ws):
+        O = torch.full_like(q, float("nan"))
+        mass = torch.empty(q.shape[:3], device=H.dev()) if with_mass else None
+        ws = sonic.sonic_attn_decode(q, K, V, H.i32(lens), O, kv_start=H.i32(starts),
+                                     max_len=int(lens.max()), chunk_len=chunk_len, workspace=ws,
+                                     role=role if with_mass else None, nexus_mass=mass)
+        torch.cuda.synchronize()
+        return O, mass, ws
+
+    O, mass, ws = run(None)
+    buf = torch.full((offset + ws.numel() + 512,), 0xA5, dtype=torch.uint8, device=H.dev())
+    part = buf[offset:offset + ws.numel()]
+    O2, mass2, used = run(part)
+    assert used.data_ptr() == part.data_ptr() == buf.data_ptr() + offset
+    assert torch.equal(O.view(torch.int16), O2.view(torch.int16))
+    assert not with_mass or torch.equal(mass, mass2)
+    assert (buf[:offset] == 0xA5).all() and (buf[offset + ws.numel():] == 0xA5).all()
