@@ -344,6 +344,9 @@ routed_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
         tma_prefetch_desc(&tmW);
         tma_prefetch_desc(&tmWn);
     }
+    // (read once for all warps: ones that saw the status differently would leave copies
+    // undrained; the partition kernels never set it)
+    if (tid == 64) misc[3] = timed_out(p.status);
     tc_fence_before();
     cluster_sync_all();  // both CTAs' barriers and tensor memory are set up
     tc_fence_after();
@@ -368,7 +371,7 @@ routed_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
     const int n0 = plain ? p.T - nx : p.groups[0], n1 = plain ? nx : p.groups[1];
     const int mt0 = (n0 + kGBM - 1) / kGBM, mt1 = (n1 + kGBM - 1) / kGBM;
     const int total_m = mt0 + mt1;
-    const int n_tiles = timed_out(p.status) ? 0 : total_m * p.n_tiles_n;
+    const int n_tiles = misc[3] ? 0 : total_m * p.n_tiles_n;
     const uint32_t tmem = static_cast<uint32_t>(misc[0]);
 
     int issued = 0;  // pipeline stages this CTA's producer filled (for the drain)
@@ -605,13 +608,14 @@ routed_small_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_consta
             if (b) kinds |= 2;
             if (lane == 0) nx_bits[w] = b;
         }
-        if (lane == 0) misc[2] = (int32_t)kinds;
+        // (the status read once: warps that saw it differently would leave copies undrained)
+        if (lane == 0) misc[2] = timed_out(p.status) ? 0 : (int32_t)kinds;
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = static_cast<uint32_t>(misc[0]);
-    const int kinds = timed_out(p.status) ? 0 : misc[2];
+    const int kinds = misc[2];
     const int n_it = (kinds == 3 ? 2 : kinds ? 1 : 0) * kbn;  // stages of the whole call
 
     int issued = 0;

@@ -213,3 +213,26 @@ def test_prefill_split_blocks_without_a_key_tile(hq, hkv, D, n):
             np.testing.assert_allclose(H.f64(lse[0]), H.f64(res["lse"][l]), rtol=0, atol=2e-3)
             np.testing.assert_allclose(H.f64(mass[0]), H.f64(res["mass"][l]), rtol=0, atol=2e-3)
         assert all(torch.equal(a, b) for a, b in zip(first[l], got))
+
+
+@pytest.mark.parametrize("T", [7, 150, 300, 2500])
+@pytest.mark.parametrize("role", [inputs.ROLE_CURR, None])
+def test_routed_linear_after_a_timeout(T, role):
+    """A status word that says a wait ran out: no block starts work (whatever the block's warps do,
+    they decide it from one read of the word), nothing is written; the next call is whole."""
+    roles = _roles(T, T) if role is None else np.full(T, role, np.uint8)
+    X = inputs.randn((T, 512), seed=1, device=H.dev())
+    W = inputs.randn((320, 512), seed=2, device=H.dev())
+    rt = torch.from_numpy(roles).to(H.dev())
+    Y = torch.full((T, 320), float("nan"), dtype=torch.bfloat16, device=H.dev())
+    status = torch.full((1,), 5, dtype=torch.int32, device=H.dev())  # SONIC_ERR_DEVICE_TIMEOUT
+    ws = sonic.sonic_routed_linear(X, W, W, rt, [(Y, False)], status=status)
+    torch.cuda.synchronize()
+    assert sonic.read_status(status) == 5 and Y.isnan().all()
+    status.zero_()
+    sonic.sonic_routed_linear(X, W, W, rt, [(Y, False)], status=status, workspace=ws)
+    torch.cuda.synchronize()
+    assert sonic.read_status(status) == 0
+    want = X.float() @ W.float().T
+    # fp32 sums of 512 products of N(0, 1) values (rms 23), rounded to bf16
+    assert ((Y.float() - want).abs() <= 2.0 ** -8 * want.abs() + 0.1).all()
