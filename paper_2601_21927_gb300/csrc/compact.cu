@@ -32,12 +32,19 @@ namespace {
 
 constexpr int kScanThreads = 512;
 constexpr int kChunks = 64;  // pieces per sequence in the scans
-// the single-launch scan (keep_plan): its largest call (rows; rows x sequences, which
-// bounds what a block counts where sequences share rows), and rows per piece
+// the single-launch scan (keep_plan): its largest call (rows; rows x sequences, as every
+// block looks at the sequences before its own), and rows per piece
 constexpr int kPlanRows = 1 << 19;
 constexpr int64_t kPlanWork = 1 << 25;
 constexpr int kPlanRowsPerThread = 4;
-constexpr int kPlanStep = kScanThreads * kPlanRowsPerThread;  // rows per piece, mostly
+constexpr int kPlanStep = kScanThreads * kPlanRowsPerThread;  // rows per piece, at least
+// rows of a long sequence's pieces; those of the others reach twice as many (where all rows are
+// more than half of kPlanRows, both are twice that: a block reads up to all role bytes, at its
+// SM's L2 rate, so more blocks do not pay)
+__host__ __device__ constexpr int long_piece(int total) {
+    return total > kPlanRows / 2 ? 2 * kPlanStep : kPlanStep;
+}
+constexpr int kSlice = 512;  // rows per slice where sequences share rows (or twice that)
 
 // Rows of sequence (start, len), or 0 when they fall outside [0, total): such a
 // sequence is refused, keeps nothing and is never read.
@@ -220,7 +227,132 @@ __device__ __forceinline__ int count_kept(const uint8_t *p, int n, int lane, int
 // sequence of 100k rows, 95.5 / 78.7 for 32 of 3k, 212 / 185 for 64 of 4k and 71.3 / 69.4 for two
 // of 250k: the line lies where the gain has run out (the counted bytes grow with the
 // square of the rows).
-// blockIdx = (piece, sequence); gridDim.x pieces per sequence.
+// One long sequence among 63 of 300 rows (three launches / this): 100k rows 37 / 13, 450k
+// 43-55 / 29-36.  Sequences that share rows: 16 that share 30k 27 / 23, 64 that share 500k
+// 859 / 826, of which the copy most.
+// blockIdx = (piece, sequence); gridDim.x pieces per sequence, enough for the mean length (the
+// host does not know the others).  One whose pieces would be longer than twice long_piece rows
+// is cut into pieces of that many, and helpers (the rows of blocks past the sequences') take
+// those past gridDim.x.  The two rare parts are functions of their own: inlined, they cost
+// every call 0.3 us or more.
+
+struct PlanShared {
+    int total[2][kScanThreads / 32];
+    int rows[kScanThreads / 32], from[kScanThreads / 32], to[kScanThreads / 32];
+    int slice[kScanThreads + 1];
+    int4 mine;  // a helper's sequence (-1: none), piece of it, its first row, its rows
+};
+
+// Rows per piece of the long sequences, and a helper's piece (to sh.mine).
+__device__ __noinline__ int32_t long_pieces(const int32_t *k_start, const int32_t *k_len, int32_t B,
+                                            int32_t total, PlanShared &sh) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int n_pieces = gridDim.x, helpers = ((int)gridDim.y - B) * n_pieces;
+    const int helper = ((int)blockIdx.y - B) * n_pieces + (int)blockIdx.x;  // (< 0: none)
+    if (tid == 0) sh.mine.x = -1;
+    for (int32_t rows = long_piece(total);; rows *= 2) {
+        int sum = 0;
+        for (int i0 = 0, k = 0; i0 < B; i0 += kScanThreads, k ^= 1) {
+            const int i = i0 + tid;
+            const int32_t s = i < B ? k_start[i] : 0, n = i < B ? seq_rows(s, k_len[i], total) : 0;
+            // its pieces that helpers take
+            const int v =
+                n > 2 * long_piece(total) * n_pieces ? max(0, (n - 1) / rows + 1 - n_pieces) : 0;
+            const int incl = warp_inclusive_scan(v);
+            if (lane == 31) sh.total[k][warp] = incl;
+            __syncthreads();
+            int at = sum + incl - v;
+            for (int w = 0; w < kScanThreads / 32; ++w) {
+                const int t = sh.total[k][w];
+                if (w < warp) at += t;
+                sum += t;
+            }
+            if (helper >= at && helper < at + v) sh.mine = make_int4(i, n_pieces + helper - at, s, n);
+        }
+        __syncthreads();
+        if (sum <= helpers) {
+            if (helper >= sum && tid == 0) sh.mine.x = -1;
+            __syncthreads();
+            return rows;
+        }
+        // (sequences that share rows have more pieces than one array of rows: longer ones)
+    }
+}
+
+// Rows kept by the first b sequences where these are not packed, this thread's share.
+__device__ __noinline__ int count_apart(const uint8_t *role, const int32_t *k_start,
+                                        const int32_t *k_len, int b, int32_t total, PlanShared &sh) {
+    constexpr int kWarps = kScanThreads / 32;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    int32_t listed = 0, from = total, to = 0;  // their rows (at most kPlanWork), in [from, to)
+    for (int i = tid; i < b; i += kScanThreads) {
+        const int32_t s = k_start[i], n = seq_rows(s, k_len[i], total);
+        listed += n;
+        from = n > 0 ? min(from, s) : from;
+        to = n > 0 ? max(to, s + n) : to;
+    }
+    listed = __reduce_add_sync(0xffffffffu, listed);
+    from = __reduce_min_sync(0xffffffffu, from);
+    to = __reduce_max_sync(0xffffffffu, to);
+    if (lane == 0) {
+        sh.rows[warp] = listed;
+        sh.from[warp] = from;
+        sh.to[warp] = to;
+    }
+    __syncthreads();
+    listed = 0;
+    for (int w = 0; w < kWarps; ++w) {
+        listed += sh.rows[w];
+        from = min(from, sh.from[w]);
+        to = max(to, sh.to[w]);
+    }
+    int kept = 0;
+    if (listed <= 2 * (to - from) + 4 * kSlice * b) {  // (few rows shared, or short sequences)
+        int wps = kWarps;  // several warps a sequence while there are few
+        while (wps > 1 && wps * b > kWarps) wps >>= 1;
+        for (int i = warp / wps; i < b; i += kWarps / wps) {
+            const int32_t s = k_start[i], n = seq_rows(s, k_len[i], total);
+            kept += count_kept(role + s, n, (warp % wps) * 32 + lane, wps * 32);
+        }
+        return kept;
+    }
+    // sequences that share rows: the rows they span are counted once, in slices, and a
+    // sequence's are those before its end less those before its start
+    const int32_t size = to - from > kScanThreads * kSlice ? 2 * kSlice : kSlice;
+    const int32_t used = (to - from + size - 1) / size;  // <= kScanThreads
+    for (int k0 = warp; k0 < used; k0 += 4 * kWarps) {
+        int n[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int32_t at = from + (k0 + j * kWarps) * size;
+            n[j] = at < to ? count_kept(role + at, min(size, to - at), lane, 32) : 0;
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            n[j] = __reduce_add_sync(0xffffffffu, n[j]);
+            if (lane == 0 && k0 + j * kWarps < used) sh.slice[k0 + j * kWarps] = n[j];
+        }
+    }
+    __syncthreads();
+    const int incl = warp_inclusive_scan(tid < used ? sh.slice[tid] : 0);
+    if (lane == 31) sh.total[0][warp] = incl;
+    __syncthreads();
+    int base = 0;
+    for (int w = 0; w < warp; ++w) base += sh.total[0][w];
+    sh.slice[tid + 1] = base + incl;  // kept rows before slice tid + 1
+    if (tid == 0) sh.slice[0] = 0;
+    __syncthreads();
+    auto upto = [&](int32_t x) {  // kept rows in [from, x), this lane's share
+        const int32_t k = (x - from) / size, at = from + k * size;
+        return (lane == 0 ? sh.slice[k] : 0) + count_kept(role + at, x - at, lane, 32);
+    };
+    for (int i = warp; i < b; i += kWarps) {
+        const int32_t s = k_start[i], n = seq_rows(s, k_len[i], total);
+        if (n > 0) kept += upto(s + n) - upto(s);
+    }
+    return kept;
+}
+
 __global__ void __launch_bounds__(kScanThreads)
 keep_plan_kernel(const uint8_t *role, const int32_t *seg,
                  const int32_t *k_start, const int32_t *k_len,
@@ -230,12 +362,29 @@ keep_plan_kernel(const uint8_t *role, const int32_t *seg,
                  int32_t *out_seg, int32_t *status) {
     pdl_wait();
     pdl_trigger();
-    const int c = blockIdx.x, b = blockIdx.y, pieces = gridDim.x;
+    const int pieces = gridDim.x;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     constexpr int kWarps = kScanThreads / 32;
+    __shared__ PlanShared sh;
     __shared__ long long seq_part[kWarps];
     __shared__ int own_part[kWarps], warp_tot[kWarps];
-    const int32_t start = k_start[b], len_in = k_len[b], first = k_start[0];
+    int c = blockIdx.x, b = min((int)blockIdx.y, B - 1);
+    int32_t start = k_start[b];
+    const int32_t len_in = k_len[b], first = k_start[0];
+    int32_t len = seq_rows(start, len_in, total);
+    int32_t rows = ((len + pieces - 1) / pieces + 31) & ~31;
+    if (blockIdx.y >= B || rows > 2 * long_piece(total)) {
+        rows = long_pieces(k_start, k_len, B, total, sh);
+        if (blockIdx.y >= B) {
+            b = sh.mine.x;
+            c = sh.mine.y;
+            start = sh.mine.z;
+            len = sh.mine.w;
+            if (b < 0) return;
+        }
+    }
+    const int32_t lo = min(len, c * rows), hi = min(len, lo + rows);
+    if (c > 0 && lo >= len) return;
     // sequences packed one after another (as a batch's mostly are) are counted as one run
     bool packed = true;
     long long before = 0;
@@ -244,10 +393,7 @@ keep_plan_kernel(const uint8_t *role, const int32_t *seg,
         packed = packed && s >= 0 && n >= 0 && (int64_t)s + n <= total && s + n == k_start[i + 1];
         if (reserve != nullptr) before += reserve[i];
     }
-    const int32_t len = seq_rows(start, len_in, total);
     if (c == 0 && tid == 0 && len != len_in) set_status(status, SONIC_ERR_INVALID_ARGUMENT);
-    const int32_t rows = ((len + pieces - 1) / pieces + 31) & ~31;
-    const int32_t lo = min(len, c * rows), hi = min(len, lo + rows);
     // this thread's rows of the piece's first step, loaded ahead of the counts
     int32_t t0 = lo + tid * kPlanRowsPerThread;
     int ro[kPlanRowsPerThread], sg[kPlanRowsPerThread + 1];
@@ -265,12 +411,7 @@ keep_plan_kernel(const uint8_t *role, const int32_t *seg,
     if (__syncthreads_and(packed)) {
         if (b > 0) before += count_kept(role + first, start - first, tid, kScanThreads);
     } else {
-        int wps = kWarps;  // several warps a sequence while there are few
-        while (wps > 1 && wps * b > kWarps) wps >>= 1;
-        for (int i = warp / wps; i < b; i += kWarps / wps) {
-            const int32_t s = k_start[i], n = seq_rows(s, k_len[i], total);
-            before += count_kept(role + s, n, (warp % wps) * 32 + lane, wps * 32);
-        }
+        before += count_apart(role, k_start, k_len, b, total, sh);
     }
     int own = count_kept(role + start, lo, tid, kScanThreads);
 #pragma unroll
@@ -327,7 +468,7 @@ keep_plan_kernel(const uint8_t *role, const int32_t *seg,
     }
     if (__syncthreads_or(bad) && tid == 0) set_status(status, SONIC_ERR_LAYOUT);
     if (c == 0 && tid == 0) offsets[b] = (int32_t)seq_base;
-    if (c != pieces - 1) return;
+    if (hi < len) return;
     // the sequence's last piece: its retained length, its reserve rows (no source), and
     // behind the last sequence the total
     const int32_t res = reserve != nullptr ? reserve[b] : 0;
@@ -479,9 +620,18 @@ extern "C" sonic_status_t sonic_compact_kv(const void *K, const void *V, const i
 
     cudaError_t e = cudaSuccess;
     if (a->total_rows <= kPlanRows && (int64_t)a->total_rows * a->batch <= kPlanWork) {
-        const int rows = a->total_rows / a->batch;
-        const int n = std::min(kChunks, std::max(1, (rows + kPlanStep - 1) / kPlanStep));
-        e = launch_pdl(keep_plan_kernel, dim3(n, a->batch), kScanThreads, 0, stream, 1, role, seg_id,
+        // pieces per sequence by the mean length, and helpers for longer ones where there can be
+        // such: enough for one array of rows, and up to a block per SM where sequences share rows
+        // (near 65,535 sequences, the grid's limit, there is no room for them: fewer pieces)
+        const int mean = a->total_rows / a->batch;
+        const int n = std::min(kChunks, std::max(1, (mean + kPlanStep - 1) / kPlanStep));
+        const bool any = a->total_rows > 2 * long_piece(a->total_rows) * n;
+        const int64_t packed = any ? a->total_rows / kPlanStep : 0;
+        const int64_t helpers =
+            std::max(packed, std::min<int64_t>(packed * a->batch, device_sm_count()));
+        const int64_t y = std::min<int64_t>(65535, a->batch + (helpers + n - 1) / n);
+        e = launch_pdl(keep_plan_kernel, dim3(n, (unsigned)std::max<int64_t>(y, a->batch)),
+                       kScanThreads, 0, stream, 1, role, seg_id,
                        a->k_start, a->k_len, a->reserve, a->batch, a->out_capacity_rows,
                        a->total_rows, offsets, a->ret_len, src_idx, a->out_role, a->out_seg,
                        a->status);

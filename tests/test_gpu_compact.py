@@ -183,3 +183,47 @@ def test_sequence_outside_the_rows_is_refused():
     keep = np.nonzero(batch.role[:int(batch.k_len[0])] != inputs.ROLE_BODY)[0]
     assert torch.equal(oK.view(torch.int16), K[:, torch.as_tensor(keep).long().to(H.dev())]
                        .view(torch.int16))
+
+
+class _Layout:
+    """Sequences given as rows [k_start, k_start + k_len) of one array of n rows."""
+    dialogues = ()
+
+    def __init__(self, n, k_start, k_len, seed):
+        rng = np.random.default_rng(seed)
+        self.role = np.repeat(rng.choice([0, 1, 1, 1, 1, 2, 3], n // 5 + 1), 5)[:n].astype(np.uint8)
+        self.seg = (np.arange(n) // 100 + 1).astype(np.int32)
+        self.k_start, self.k_len = np.asarray(k_start, np.int32), np.asarray(k_len, np.int32)
+        self.B = len(self.k_start)
+
+
+def _layouts():
+    rng = np.random.default_rng(3)
+    for n_seqs in (2, 9, 17, 100):
+        lens = rng.integers(0, 2 * 5000 // (1 + n_seqs // 20), n_seqs)
+        at = np.concatenate([[0], np.cumsum(lens)])
+        n = int(at[-1])
+        long1 = np.r_[150_000, rng.integers(0, 300, n_seqs - 1)]
+        rng.shuffle(long1)
+        lstart = np.r_[0, np.cumsum(long1)[:-1]]
+        yield f"long{n_seqs}", int(long1.sum()), lstart, long1
+        gap = rng.integers(0, 90, n_seqs)
+        yield f"gaps{n_seqs}", n + int(gap.sum()), at[:-1] + np.cumsum(gap), lens
+        yield f"down{n_seqs}", n, at[:-1][::-1], lens[::-1]
+        yield f"same{n_seqs}", 30_001, np.zeros(n_seqs, int), np.full(n_seqs, 30_001)
+        s = rng.integers(0, 20_000, n_seqs)
+        yield f"shared{n_seqs}", 40_000, s, rng.integers(0, 40_000 - s)
+
+
+@pytest.mark.parametrize("name,n,k_start,k_len", list(_layouts()), ids=lambda v: v if type(v) is str else "")
+def test_layouts_of_sequences(name, n, k_start, k_len):
+    """One long sequence among short ones, gaps between sequences, starts in descending order, and
+    sequences that share all or part of their rows: offsets, lengths, sources, roles, segments and
+    bytes; with and without reserve rows."""
+    lay = _Layout(n, k_start, k_len, len(k_start))
+    K = inputs.randn((1, n, 1, 8), seed=n, device=H.dev())
+    V = inputs.randn((1, n, 1, 8), seed=n + 1, device=H.dev())
+    for reserve in (None, np.arange(lay.B) % 4):
+        off, _, _ = oracle.retain(lay.k_start, lay.k_len, lay.role, reserve)
+        r = _run(lay, K, V, reserve=reserve, cap=int(off[-1]))
+        _check(lay, K, V, r, reserve=reserve)
