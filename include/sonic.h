@@ -366,7 +366,8 @@ typedef struct {
     int32_t n_parts;             /* 1 .. 4                                              */
     sonic_out_part parts[4];
     int32_t *status;             /* device int32 or NULL                                */
-    void *workspace;             /* device, sonic_routed_linear_workspace_size() bytes  */
+    void *workspace;             /* device, sonic_routed_linear_workspace_size() bytes,
+                                    16-byte aligned                                     */
     size_t workspace_bytes;
 } sonic_routed_linear_args;
 

@@ -848,6 +848,8 @@ extern "C" sonic_status_t sonic_routed_linear(const uint16_t *X, const uint16_t 
     if ((long long)a->n_rows * a->d_in > (1LL << 40)) return SONIC_ERR_UNSUPPORTED;
     const RlWorkspace ws = rl_workspace(a);
     if (a->workspace == nullptr || a->workspace_bytes < ws.total) return SONIC_ERR_WORKSPACE;
+    // (TMA reads the grouped rows there; refused for calls of few rows too, which leave it unused)
+    if (!aligned16(a->workspace)) return SONIC_ERR_INVALID_ARGUMENT;
 
     char *wsb = static_cast<char *>(a->workspace);
     int32_t *counts = reinterpret_cast<int32_t *>(wsb + ws.counts);

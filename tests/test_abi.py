@@ -178,3 +178,12 @@ def test_decode_workspace_has_room_for_any_alignment():
     d.batch, d.n_layers, d.n_heads_q, d.n_heads_kv, d.head_dim = 2, 1, 8, 2, 128
     d.max_len, d.total_kv_rows, d.chunk_len = 10, 20, 128
     assert lib.sonic_decode_workspace_size(ctypes.byref(d)) == 256 + 16
+
+
+def test_routed_linear_refuses_a_misaligned_workspace():
+    lib = sonic.load()
+    a = sonic.sonic_routed_linear_args()
+    a.n_rows, a.d_in, a.d_out, a.x_row_stride, a.n_parts = 10, 128, 64, 128, 1
+    a.parts[0].base, a.parts[0].row_stride, a.parts[0].cols, a.parts[0].rows = 16, 64, 64, 10
+    a.workspace, a.workspace_bytes = 24, 1 << 20
+    assert lib.sonic_routed_linear(16, 16, 16, 16, ctypes.byref(a), None) == 1

@@ -236,3 +236,22 @@ def test_routed_linear_after_a_timeout(T, role):
     want = X.float() @ W.float().T
     # fp32 sums of 512 products of N(0, 1) values (rms 23), rounded to bf16
     assert ((Y.float() - want).abs() <= 2.0 ** -8 * want.abs() + 0.1).all()
+
+
+@pytest.mark.parametrize("T", [1, 16, 192, 193, 700])
+def test_routed_linear_refuses_a_misaligned_workspace(T):
+    """Refused whatever the number of rows, also where the call has no use for the workspace."""
+    X = inputs.randn((T, 128), seed=1, device=H.dev())
+    W = inputs.randn((64, 128), seed=2, device=H.dev())
+    role = torch.full((T,), inputs.ROLE_CURR, dtype=torch.uint8, device=H.dev())
+    Y = torch.full((T, 64), float("nan"), dtype=torch.bfloat16, device=H.dev())
+    ws = sonic.sonic_routed_linear(X, W, W, role, [(Y, False)])
+    Y.fill_(float("nan"))
+    buf = torch.empty(ws.numel() + 16, dtype=torch.uint8, device=H.dev())
+    assert buf.data_ptr() % 16 == 0
+    for offset in (1, 8):
+        with pytest.raises(sonic.SonicError) as e:
+            sonic.sonic_routed_linear(X, W, W, role, [(Y, False)], workspace=buf[offset:])
+        assert e.value.code == 1
+    torch.cuda.synchronize()
+    assert Y.isnan().all()
