@@ -61,12 +61,14 @@ struct TileSum {
     int32_t pos_max;
 };
 
-// Calls of several units per block claim their sequences by length, the longest first:
-// a unit's time grows with its keys (98 key tiles are ~170 us), and claimed late it is
-// what the call ends on.  (Sequences within 1.5 x of one another keep their order: by
-// length four of 2.1-2.9k keys took 160 us instead of 149, as it happens to fall, with
-// nothing to gain on the average.)  The order (a byte per sequence) sits behind the unit counter in
-// its 256 bytes of workspace, so up to kSeqOrder sequences; more keep their given order.
+// Calls of several unpaired or single-tile units per block claim their sequences by length, the
+// longest first (sequences within 1.5 x of one another keep their order).  100 ragged sequences
+// of four layers and 28/4 heads, units of 3 to 6 key tiles, took 674 us in the given order and
+// 552 by length; 40 of two layers 172 and 158; 30 single-tile ones of four layers 96 and 88.
+// Paired units keep the given order: by length six turns of 190-1,500 rows took 149 us
+// instead of 134, seven of 156-306 rows 63 instead of 55, eight long ones 1,390 instead of
+// 1,397.  The order (a byte per sequence) sits behind the unit counter in its 256 bytes of
+// workspace, so up to kSeqOrder sequences; more keep their given order.
 constexpr int kSeqOrder = 252;
 
 // Key rows with role 255 are padding (no key): they count as invalid.
@@ -593,8 +595,17 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     uint64_t *k_empty = bars + 26;  // [3]
     uint64_t *pv_done = bars + 29;
     int32_t *misc = reinterpret_cast<int32_t *>(smem + C::kOffMisc);
-    // misc: 0 tmem base, 2 abort, 3 the scheduler copied the first unit's Q
+    // misc: 0 tmem base, 1 key tiles copied (kLate), 2 abort, 3 the scheduler copied the first
+    // unit's Q
     volatile int *abort_flag = reinterpret_cast<volatile int *>(misc + 2);
+    // A block claims its next unit when few of the current one's key tiles are left to copy: as
+    // many as take the time in which a list is made (the claim and its loads, and a look at 32
+    // tile summaries per round).  Claimed as soon as the scheduler was free, up to two units
+    // ahead, the units of a call of a few per block went to whichever blocks were quickest at the
+    // start: four ragged turns of up to 700 rows (28/4 heads) took 75-89 us, now 69; one
+    // of 1,500 rows 90, now 78; six turns of up to 1,500 rows (8/2 heads) 66-76, now 56.
+    constexpr bool kLate = !kQC && !kSplit && !kSolo;
+    volatile int *tiles_issued = reinterpret_cast<volatile int *>(misc + 1);
 
     // A query tile is R query rows x P heads of one KV group (P = 1 << pack_log2,
     // R = 128 / P): tile row r is query row r / P, head h0 + r % P.  P > 1 packs
@@ -633,6 +644,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
             mbar_init(pv_done, 1);
         }
         *abort_flag = 0;
+        if (kLate) *tiles_issued = 0;
         if (!kQC) misc[3] = 0;
         fence_mbar_init();
         if (!kQC) {
@@ -671,8 +683,15 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         // ------------------------------------------------------------ scheduler
         bool taken = false;  // the block's first unit is taken
         bool waited = !kEarly;  // the kernel before this one is complete
+        int listed = 0;  // kLate: key tiles of the units so far
         for (int k = 0;; ++k) {
             const int slot = k & 1;
+            if (kLate && k > 0) {
+                const uint64_t t0 = global_ns();
+                while (listed - *tiles_issued > 4 + (p.max_k_tiles >> 5) && !*abort_flag &&
+                       global_ns() - t0 < SONIC_WAIT_LIMIT_NS)
+                    __nanosleep(200);
+            }
             int end = 0, layer = 0, b = 0, hg = 0, qt = 0, cw = 0;
             bool lpair = false;  // a last query block shared by two heads (below)
             int kstart = 0, klen = 0, qstart = 0, qlen = 0, kkstart = 0, kklen = 0;
@@ -683,7 +702,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                     if (lane == 0 && !*abort_flag && !timed_out(p.status)) u = atomicAdd(p.counter, 1);
                     u = __shfl_sync(0xffffffffu, u, 0);
                 } else if (!taken) {
-                    if (!waited && !kSplit && p.seq_order != nullptr) {
+                    if (kSolo && !kSplit && !waited && p.seq_order != nullptr) {
                         pdl_wait();  // (the summary kernel writes it)
                         waited = true;
                     }
@@ -708,7 +727,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                 int rest = u / p.HG;
                 qt = p.qtiles - 1 - rest % p.qtiles;
                 rest /= p.qtiles;
-                if (!kQC && !kSplit && p.seq_order != nullptr) {
+                if (!kQC && !kPair && !kSplit && p.seq_order != nullptr) {
                     layer = rest % p.n_layers;
                     b = p.seq_order[rest / p.n_layers];
                 } else {
@@ -952,6 +971,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                 if (b1) last1 = n_list + __popc(bal & ((2u << (31 - __clz(b1))) - 1u)) - 1;
                 n_list += __popc(bal);
             }
+            if (kLate) listed += n_list;
             // both query tiles visit every listed key tile (masked where they see
             // none of it) unless skipping drops more than a tenth of the products
             const bool dense = kSplit || skipped * 10 <= (tile1 ? 2 : 1) * n_list;
@@ -1191,6 +1211,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                                         layer);
                             tma_load_5d(Vs + st * C::kKVBytes, mv, &kv_full[st], 0, kvh, row, 0,
                                         layer);
+                            if (kLate) *tiles_issued = g + 1;
                         }
                         issued_kv = g + 1;
                         stage_meta(st, e, need_m0, need_m1);
@@ -2560,12 +2581,10 @@ extern "C" sonic_status_t sonic_attn_prefill(const uint16_t *Q, const uint16_t *
     const bool solo = !qchunked && pack_log2 > 0 && a->max_q_len <= R;
     // one persistent block per SM (fewer when there are fewer units)
     const int grid = (int)std::min<long long>(device_sm_count(), n_units);
-    // several units per block: sequences claimed by length (GPU time, given order / by
-    // length: eight resuming sequences of 3-12.6k keys, one layer 736 / 706 us, six ragged
-    // ones of two layers 381 / 351, ten shorter ones 135 / 111; layers innermost, so that the
-    // shortest of all layers come last: layer by layer the six took 380).  Single-tile units
-    // start before the order is written, which is worth more to a few.
-    const bool by_len = !qchunked && a->batch > 1 && a->batch <= kSeqOrder && n_units > (solo ? 4LL * grid : grid);
+    // sequences claimed by length (see kSeqOrder); single-tile units start before the order is
+    // written, which is worth more to a few
+    const bool by_len = !qchunked && !pair && a->batch > 1 && a->batch <= kSeqOrder &&
+                        n_units > (solo ? 4LL * grid : grid);
     uint8_t *order = by_len ? reinterpret_cast<uint8_t *>(p.counter) + 4 : nullptr;
     p.seq_order = order;
     cudaError_t e = launch_pdl(

@@ -342,3 +342,29 @@ def test_longest_sequence(order, L):
     O, lse, got, got_lse = H.oracle_prefill_rows(batch, res, 0, np.array([0, 31, 63]))
     H.check_close(got, O, "longest sequence")
     np.testing.assert_allclose(got_lse, lse, rtol=0, atol=2e-3)
+
+
+@pytest.mark.parametrize("hq,hkv,D,most", [(8, 2, 128, 700), (6, 2, 128, 500), (28, 4, 64, 40),
+                                           (8, 2, 64, 30), (7, 1, 128, 300)])
+def test_ragged_batch_of_several_units_per_block(hq, hkv, D, most):
+    """Paired, unpaired and single-tile units, several per block, claimed one after another: ragged
+    sequences of 1 to 24 key tiles with up to `most` query rows, some with none."""
+    rng = np.random.default_rng(hq + D)
+    ds = [inputs.Dialogue(int(rng.integers(1, 300)),
+                          [(int(rng.integers(0, 200)), int(rng.integers(0, 40)))
+                           for _ in range(int(rng.integers(0, 12)))], int(rng.integers(1, 800)))
+          for _ in range(26)]
+    batch = inputs.Batch(ds)
+    q_len = np.minimum(batch.k_len, rng.integers(1, most + 1, batch.B)).astype(np.int32)
+    q_len[rng.integers(0, batch.B, 3)] = 0
+    res = H.run_prefill(batch, hq, hkv, D, q_len=q_len, n_layers=3, seed=hq, with_mass=True)
+    assert torch.isfinite(res["O"]).all()
+    for b in range(0, batch.B, 3):
+        if q_len[b] == 0:
+            continue
+        rows = np.unique(np.r_[0, q_len[b] // 2, q_len[b] - 1])
+        O, lse, got, got_lse = H.oracle_prefill_rows(batch, res, b, rows, layer=2)
+        H.check_close(got, O, f"seq {b}")
+        np.testing.assert_allclose(got_lse, lse, rtol=0, atol=2e-3)
+        want, mass = H.oracle_mass_rows(batch, res, b, rows, layer=2)
+        np.testing.assert_allclose(mass, want, rtol=0, atol=2e-3)
