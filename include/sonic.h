@@ -384,8 +384,8 @@ typedef struct {
  * the rows compaction reserved), so new tokens' keys and values land in the
  * retained cache with no further copy.  Rows are grouped by role on the GPU
  * (a stable partition, no host round trip) and the GEMM runs on the tensor
- * cores; the workspace holds the grouped copy of X (calls of at most 192 rows
- * need no grouping and leave it unused).  T = 0 does nothing.
+ * cores; the workspace holds the grouped copy of X (calls of few rows, at most
+ * 192, need no grouping and leave it unused).  T = 0 does nothing.
  */
 SONIC_API sonic_status_t sonic_routed_linear(const uint16_t *X, const uint16_t *W,
                                              const uint16_t *W_nexus, const uint8_t *role,

@@ -557,7 +557,14 @@ struct SmallCfg {
                                           : NT <= 128 ? 256 : 512;
 };
 
-constexpr int kSmallRows = 192;
+// Largest T of it: what is said above holds where the weight tiles take clusters of two or
+// more.  With one CTA per tile every tile's whole reduction reads all of X (8192 -> 10240, GPU time
+// in us, this / pair tiles: 44.2 / 48.0 at 128 rows, 55.5 / 48.1 at 160), and with more tiles than
+// SMs in two waves (4096 -> 20480: 46.5 / 49.6 at 16 rows, but 86 / 76 at 32 of both kinds).
+int small_rows(int d_out) {
+    const int tiles = (d_out + kHalfN - 1) / kHalfN, sms = device_sm_count();
+    return 2 * tiles <= sms ? 192 : tiles <= sms ? 128 : 16;
+}
 
 template <int NT>
 __global__ void __launch_bounds__(kGThreads, 1)
@@ -883,7 +890,7 @@ extern "C" sonic_status_t sonic_routed_linear(const uint16_t *X, const uint16_t 
                : e == cudaErrorInvalidValue ? SONIC_ERR_INVALID_ARGUMENT
                                             : SONIC_ERR_CUDA;
     };
-    if (T <= kSmallRows) {
+    if (T <= small_rows(a->d_out)) {
         const auto launch = T <= 16    ? launch_small<16>
                             : T <= 32  ? launch_small<32>
                             : T <= 64  ? launch_small<64>

@@ -255,3 +255,13 @@ def test_routed_linear_refuses_a_misaligned_workspace(T):
         assert e.value.code == 1
     torch.cuda.synchronize()
     assert Y.isnan().all()
+
+
+@pytest.mark.parametrize("tiles,T", [(76, 192), (76, 193), (77, 128), (77, 129), (152, 128),
+                                     (152, 129), (153, 16), (153, 17)])
+def test_routed_linear_widths_at_the_lines(tiles, T):
+    """Both sides of the largest call of few rows, where the 128-row weight tiles take clusters, one
+    CTA each, or more than one wave (152 SMs)."""
+    d_out = tiles * 128 - 96
+    r = _run(_roles(T, T), 128, [d_out - 64, 64], [False, True], seed=tiles, cache_rows=T + 3)
+    _check(r)
