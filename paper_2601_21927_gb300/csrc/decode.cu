@@ -834,53 +834,12 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     if (warp == 1) tmem_dealloc(tmem, kTmemCols);
 }
 
-// One warp per (layer, sequence, query head): the log-sum-exp merge of its pieces
-// (chunks, or the shares its sequence is cut into).  A warp's lanes fetch the pieces'
-// maxima and sums side by side, then every accumulator load is independent of them.
+// One (layer, sequence, query head): its n pieces (none: zeros), by one warp.
 template <int D>
-__global__ void __launch_bounds__(128)
-decode_combine_kernel(const DecParams p, int n_layers) {
-    // The main kernel lets this one start once everything ahead of the call is complete, so
-    // the lengths are read and the pieces found while it still runs (1.0-1.5 us less behind
-    // every call: 1 x 641 rows 10.8 -> 9.8 us, 16 x 641 19.9 -> 18.8).
-    const int64_t unit = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+__device__ __forceinline__ void combine_head(const DecParams &p, int b, int layer, int h, int n,
+                                             int64_t slot0, int64_t slot1, int64_t step) {
     const int lane = threadIdx.x & 31;
-    const int64_t n_units = (int64_t)n_layers * p.B * p.Hq;
-    if (unit >= n_units) {
-        pdl_wait();  // (no block ends before the main kernel: the next call reuses its workspace)
-        return;
-    }
-    const int h = (int)(unit % p.Hq);
-    const int64_t lb = unit / p.Hq;
-    const int b = (int)(lb % p.B), layer = (int)(lb / p.B);
-    const int len = seq_keys(p, p.lens[b], p.kv_start[b]);
-    // pieces 0 .. n - 1; the slot of piece c is slot0 (c = 0) or slot1 + c * step
-    int n = (len + p.chunk_len - 1) / p.chunk_len;
-    int64_t slot0 = unit * p.max_chunks, slot1 = slot0, step = 1;
-    if (p.groups > 0 && len > 0) {
-        int before = 0, sum = 0;
-        for (int i = lane; i < p.B; i += 32) {
-            const int li = seq_keys(p, p.lens[i], p.kv_start[i]);
-            sum += li;
-            before += i < b ? li : 0;
-        }
-        sum = __reduce_add_sync(0xffffffffu, sum);
-        before = __reduce_add_sync(0xffffffffu, before);
-        const int per = share_of(sum * n_layers, p.groups), s0 = layer * sum + before;
-        // first and last group with keys of this sequence: its cuts are those of the
-        // multiples of per in [s0, s0 + len)
-        const int lo = (s0 + per - 1) / per, hi = (s0 + len - 1) / per;
-        const int ga = lo <= hi && snap(lo * per - s0, len) == 0 ? lo : lo - 1;
-        const int gz = lo <= hi && snap(hi * per - s0, len) == len ? hi - 1 : hi;
-        const int heads = p.slot_heads, kvh = h / heads, hl = h % heads;
-        n = gz - ga + 1;
-        slot0 = (((int64_t)ga * p.Hkv + kvh) * 2 + 1) * heads + hl;  // from the sequence's start
-        step = (int64_t)p.Hkv * 2 * heads;
-        slot1 = slot0 - heads;
-    }
-    pdl_wait();
-    pdl_trigger();
-    if (n == 1) return;  // written by the split kernel
+    const int64_t unit = ((int64_t)layer * p.B + b) * p.Hq + h;
     uint16_t *op = p.O + layer * p.o_ls + ((int64_t)b * p.Hq + h) * D;
     constexpr int kDpl = D / 32;
     using Vec = typename std::conditional<kDpl == 4, float4, float2>::type;
@@ -934,8 +893,15 @@ decode_combine_kernel(const DecParams p, int n_layers) {
             c = kFirst;
         }
         const int m = min(n - c0, 32);
-#pragma unroll 8
-        for (; c < m; ++c) add(c, acc_of(c0 + c));
+        for (; c < m; c += kFirst) {
+            Vec v[kFirst];
+#pragma unroll
+            for (int k = 0; k < kFirst; ++k)
+                if (c + k < m) v[k] = acc_of(c0 + c + k);
+#pragma unroll
+            for (int k = 0; k < kFirst; ++k)
+                if (c + k < m) add(c + k, v[k]);
+        }
     }
     uint32_t w[kDpl / 2];
 #pragma unroll
@@ -944,6 +910,88 @@ decode_combine_kernel(const DecParams p, int n_layers) {
     for (int e = 0; e < kDpl; ++e) op[lane * kDpl + e] = (uint16_t)(w[e >> 1] >> ((e & 1) * 16));
     if (lane == 0 && p.lse != nullptr) p.lse[unit] = (M + __log2f(L)) * kLn2;
     if (lane == 0 && p.nexus_mass != nullptr) p.nexus_mass[unit] = N / L;
+}
+
+// The log-sum-exp merge of a sequence's pieces (chunks, or the shares it is cut into): a block
+// per (layer, sequence, 4 * heads_per_warp query heads), a warp per head at a time.  A warp's
+// lanes fetch the pieces' maxima and sums side by side, then every accumulator load is
+// independent of them.  Where a sequence lies on the line of keys takes all lengths: each
+// warp adds them up, or (by many sequences) each block, for all heads of its sequence.  Each
+// warp of each head doing so had made calls of many short sequences slower than chunks:
+// 1,000 of 16/1 heads 54 us in chunks, 72, now 51; 700 of 28/4 82, 86, now 78.
+constexpr int kCombineThreads = 128;
+constexpr int kCombineSeqs = 256;     // sequences from which a block sums the lengths together
+constexpr int kCombineAllHeads = 512;  // and from which it takes all heads
+
+template <int D, bool kMany>  // kMany: more than kCombineSeqs sequences
+__global__ void __launch_bounds__(kCombineThreads)
+decode_combine_kernel(const DecParams p, int heads_per_warp) {
+    // The main kernel lets this one start once everything ahead of the call is complete, so
+    // the lengths are read and the pieces found while it still runs (1.0-1.5 us less behind
+    // every call: 1 x 641 rows 10.8 -> 9.8 us, 16 x 641 19.9 -> 18.8).
+    constexpr int kWarps = kCombineThreads / 32;
+    __shared__ int part[2][kWarps];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int per_block = kMany ? kWarps * heads_per_warp : kWarps;
+    const int blocks = (p.Hq + per_block - 1) / per_block;
+    const int64_t lb = blockIdx.x / blocks;
+    const int b = (int)(lb % p.B), layer = (int)(lb / p.B);
+    const int len = seq_keys(p, p.lens[b], p.kv_start[b]);
+    // pieces 0 .. n - 1, the first of them in group ga
+    int n = (len + p.chunk_len - 1) / p.chunk_len, ga = 0;
+    if (p.groups > 0 && len > 0) {
+        int before = 0, sum = 0;
+        for (int i = kMany ? threadIdx.x : lane; i < p.B; i += kMany ? kCombineThreads : 32) {
+            const int li = seq_keys(p, p.lens[i], p.kv_start[i]);
+            sum += li;
+            before += i < b ? li : 0;
+        }
+        sum = __reduce_add_sync(0xffffffffu, sum);
+        before = __reduce_add_sync(0xffffffffu, before);
+        if (kMany) {
+            if (lane == 0) {
+                part[0][warp] = sum;
+                part[1][warp] = before;
+            }
+            __syncthreads();
+            sum = before = 0;
+            for (int w = 0; w < kWarps; ++w) {
+                sum += part[0][w];
+                before += part[1][w];
+            }
+        }
+        const int per = share_of(sum * p.n_layers, p.groups), s0 = layer * sum + before;
+        // first and last group with keys of this sequence: its cuts are those of the
+        // multiples of per in [s0, s0 + len)
+        const int lo = (s0 + per - 1) / per, hi = (s0 + len - 1) / per;
+        ga = lo <= hi && snap(lo * per - s0, len) == 0 ? lo : lo - 1;
+        const int gz = lo <= hi && snap(hi * per - s0, len) == len ? hi - 1 : hi;
+        n = gz - ga + 1;
+    }
+    // the slot of a head's piece c is slot0 (c = 0) or slot1 + c * step
+    const int h0 = (int)(blockIdx.x % blocks) * per_block, h1 = min(h0 + per_block, p.Hq);
+    int64_t slot0, slot1, step;
+    auto slots = [&](int h) {
+        slot0 = slot1 = ((int64_t)lb * p.Hq + h) * p.max_chunks;
+        step = 1;
+        if (p.groups > 0) {
+            const int heads = p.slot_heads, kvh = h / heads, hl = h % heads;
+            slot0 = (((int64_t)ga * p.Hkv + kvh) * 2 + 1) * heads + hl;  // from the start on
+            step = (int64_t)p.Hkv * 2 * heads;
+            slot1 = slot0 - heads;
+        }
+    };
+    int h = h0 + warp;
+    slots(h);
+    // (no block ends before the main kernel: the next call reuses its workspace)
+    pdl_wait();
+    pdl_trigger();
+    if (n == 1) return;  // written by the split kernel
+    for (; h < h1; h += kWarps) {
+        combine_head<D>(p, b, layer, h, n, slot0, slot1, step);
+        if (!kMany) break;
+        slots(h + kWarps);
+    }
 }
 
 // Every output of a call with no key rows at all: O = 0, lse = -inf, mass 0.
@@ -1011,8 +1059,16 @@ Plan make_plan(const sonic_decode_args *a) {
     size_t slots = pl.max_chunks > 1 ? units_q * pl.max_chunks : 0;
     const int sms = device_sm_count();
     const long long keys = (long long)a->n_layers * a->batch * pl.max_chunks * C;
-    if (a->chunk_len == 0 && a->batch <= TcCfg::kSeqCache && kv_units >= 1 && kv_units <= sms &&
-        sms / kv_units * kv_units * 8 >= sms * 7 && keys <= (1 << 30)) {
+    // With more than 8 query heads to a unit a tile costs the same however few keys it has, so
+    // cutting sequences is no gain where they are short or many (GPU time in us, chunks / shares:
+    // 16/1 heads, 300 of up to 200 keys 25 / 31, 1,000 of up to 900 91 / 96), nor with one KV
+    // head where they are both (2/1, 900 of 45 keys 25 / 28).
+    const long long seqs = (long long)a->batch * a->n_layers;
+    const bool brief = max_len <= 2 * kTcKeys, wide = a->n_heads_q > 8 * kv_units;
+    const bool whole = (wide && brief && seqs >= 32) ||
+                       ((wide || (brief && kv_units == 1)) && 2 * seqs * kv_units >= 5LL * sms);
+    if (a->chunk_len == 0 && !whole && a->batch <= TcCfg::kSeqCache && kv_units >= 1 &&
+        kv_units <= sms && sms / kv_units * kv_units * 8 >= sms * 7 && keys <= (1 << 30)) {
         const long long most = (keys + kMinShare - 1) / kMinShare;
         pl.groups = (int)(most < sms / kv_units ? most : sms / kv_units);
         // two partial pieces per block, of all query heads of its unit
@@ -1192,9 +1248,18 @@ extern "C" sonic_status_t sonic_attn_decode(const uint16_t *q, const uint16_t *K
                                          stream)
                  : dispatch_tc<64, false>(GT, tm, p, (int)units_x, n_units, counter, stream);
     if (e != cudaSuccess) return SONIC_ERR_CUDA;
-    const long long units = (long long)a->n_layers * a->batch * a->n_heads_q;
-    const unsigned cblocks = (unsigned)((units * 32 + 127) / 128);
-    e = launch_pdl(D == 128 ? decode_combine_kernel<128> : decode_combine_kernel<64>, dim3(cblocks),
-                   128, 0, stream, 1, p, a->n_layers);
+    const bool many = a->batch > kCombineSeqs;
+    constexpr int kWarps = kCombineThreads / 32;
+    const int heads_per_warp =
+        pl.groups > 0 && a->batch > kCombineAllHeads ? (a->n_heads_q + kWarps - 1) / kWarps : 1;
+    const int per_block = kWarps * heads_per_warp;
+    const long long cblocks = (long long)a->n_layers * a->batch *
+                              ((a->n_heads_q + per_block - 1) / per_block);
+    const auto combine = D == 128 ? (many ? decode_combine_kernel<128, true>
+                                          : decode_combine_kernel<128, false>)
+                                  : (many ? decode_combine_kernel<64, true>
+                                          : decode_combine_kernel<64, false>);
+    e = launch_pdl(combine, dim3((unsigned)cblocks), kCombineThreads, 0, stream, 1, p,
+                   heads_per_warp);
     return e == cudaSuccess ? SONIC_OK : SONIC_ERR_CUDA;
 }

@@ -246,3 +246,20 @@ def test_workspace_at_any_alignment(D, hq, chunk_len, with_mass, offset):
     assert torch.equal(O.view(torch.int16), O2.view(torch.int16))
     assert not with_mass or torch.equal(mass, mass2)
     assert (buf[:offset] == 0xA5).all() and (buf[offset + ws.numel():] == 0xA5).all()
+
+
+@pytest.mark.parametrize("hq,hkv,D,B", [(8, 2, 128, 257), (16, 1, 128, 300), (28, 4, 128, 513),
+                                        (2, 1, 64, 1024), (16, 2, 64, 1025), (16, 1, 64, 40)])
+def test_many_short_sequences(hq, hkv, D, B):
+    """More sequences than a warp adds up lengths for, than have a block of their own for each four
+    heads, and than the lengths are cached for (1,024); empty ones among them."""
+    rng = np.random.default_rng(B)
+    lens = rng.integers(0, 200, B)
+    lens[rng.integers(0, B, 5)] = 0
+    lens[rng.integers(0, B, 2)] = 700 if B > 40 else 256
+    r = _decode(lens, hq, hkv, D, n_layers=2, seed=B, pad=1, with_mass=True)
+    pairs = [(l, b) for l in (0, 1) for b in list(range(0, B, 1 + B // 25)) + [B - 1]]
+    pairs += [(1, int(b)) for b in np.flatnonzero((lens == 0) | (lens >= 256))[:8]]
+    _check(r, pairs)
+    _check_mass(r, pairs)
+    assert not r["O"].isnan().any()
