@@ -1,7 +1,8 @@
-"""Calls of a few rows, which take kernels of their own: the role-routed linear map of at
-most 192 rows (weights as the M operand, reduction split over a cluster), at the edges
-of its row paddings (16, 32, 64, 128, 192), with and without a split, ragged column
-tiles, one kind of row or both."""
+"""Calls that take kernels of their own by their size, at the edges of their ranges: the
+role-routed linear map of few rows (the row paddings 16, 32, 64, 128, 192, with and without a
+split of the reduction, ragged column tiles, one kind of row or both; the lines by width) and of
+very many; decode in equal shares; the single-launch scan of the compaction; prefills whose units
+are shared by clusters of blocks; calls captured behind copies and memsets."""
 import numpy as np
 import pytest
 import torch
@@ -34,6 +35,13 @@ def test_routed_linear_projection_widths(role, T, d_in, cols):
     roles = _roles(T, T) if role is None else np.full(T, role, np.uint8)
     r = _run(roles, d_in, cols, [False] + [True] * (len(cols) - 1), seed=41, cache_rows=T + 9)
     _check(r)
+
+
+@pytest.mark.parametrize("T", [131072, 131073])
+def test_routed_linear_counted_by_a_launch_of_its_own(T):
+    """Both sides of the largest call whose partition counts the roles itself."""
+    r = _run(_roles(T, 7), 64, [32, 32], [False, True], seed=T, cache_rows=T + 5)
+    _check(r, np.r_[0:300, T // 2:T // 2 + 300, T - 300:T])
 
 
 @pytest.mark.parametrize("T", [16384, 16385])
@@ -125,13 +133,14 @@ def test_calls_captured_after_copies_and_memsets():
         assert torch.equal(Y.view(torch.int16), want[1].view(torch.int16))
 
 
-@pytest.mark.parametrize("n_seqs,rows,total", [(1, 131072, 131072), (1, 131073, 131073),
+@pytest.mark.parametrize("n_seqs,rows,total", [(1, 524288, 524288), (1, 524289, 524289),
+                                               (128, 2048, 1 << 18), (128, 2049, 128 * 2049),
                                                (2, 2047, 0), (3, 2049, 0), (15, 900, 0),
                                                (17, 4100, 0), (40, 77, 0), (128, 300, 0)])
 def test_compact_single_launch_scan(n_seqs, rows, total):
-    """On both sides of the largest call of the single-launch scan (131,072 rows), sequences
-    at every alignment of the role bytes, pieces that end off the 16-byte words, empty
-    and body-only sequences among them, reserve rows."""
+    """On both sides of the largest calls of the single-launch scan (524,288 rows; rows x sequences
+    of 2^25), sequences at every alignment of the role bytes, pieces that end off the 16-byte
+    words, empty and body-only sequences among the ragged ones, reserve rows."""
     rng = np.random.default_rng(rows)
     ds = []
     for k in range(n_seqs):
@@ -142,7 +151,7 @@ def test_compact_single_launch_scan(n_seqs, rows, total):
             segs.append((b, x))
             left -= b + x
         ds.append(inputs.Dialogue(int(rng.integers(0, left + 1)) if not total else left, segs, 0))
-    if n_seqs > 2:
+    if n_seqs > 2 and not total:
         ds[1], ds[2] = inputs.Dialogue(0, [], 0), inputs.Dialogue(0, [(333, 0)], 0)
     batch = inputs.Batch(ds)
     assert not total or batch.total == total
