@@ -68,8 +68,8 @@ __device__ __forceinline__ bool seq_refused(const DecParams &p, int raw_len, int
 // away, so no piece is shorter than that unless its sequence is.  Claimed chunks of
 // ~1/4 of an SM's work left the SMs with up to a chunk more than others (56 ragged
 // sequences of 28/4 heads: 82 us, 4.4 TB/s; in shares 68, 5.3), and short calls with
-// a counter to clear first (16 x 641 rows: 24.4, now 18.8; 64 long ragged ones, four layers:
-// 758, 7.2 TB/s now in 694).  The explicit split (chunk_len) and batches above kSeqCache
+// a counter to clear first (16 x 641 rows: 24.5, now 17.2; 64 long ragged ones, four layers,
+// 5.0 GB: 758, now 684-695, 7.2-7.4 TB/s).  The explicit split (chunk_len) and batches above kSeqCache
 // sequences, or KV heads that leave over an eighth of the SMs without a group, keep the
 // chunks.
 constexpr int kMinShare = 64;
@@ -928,7 +928,7 @@ __global__ void __launch_bounds__(kCombineThreads)
 decode_combine_kernel(const DecParams p, int heads_per_warp) {
     // The main kernel lets this one start once everything ahead of the call is complete, so
     // the lengths are read and the pieces found while it still runs (1.0-1.5 us less behind
-    // every call: 1 x 641 rows 10.8 -> 9.8 us, 16 x 641 19.9 -> 18.8).
+    // every call: 1 x 641 rows 10.8 -> 9.8 us, 16 x 641 19.9 -> 18.8 at the time).
     constexpr int kWarps = kCombineThreads / 32;
     __shared__ int part[2][kWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;

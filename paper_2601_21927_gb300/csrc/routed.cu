@@ -4,7 +4,7 @@
 // buffers of their own, each at the row itself or at a caller-given row (so
 // the K and V of new tokens land straight in their retained-cache rows).
 //
-// At most 192 rows take one kernel, routed_small (see there).  More take these
+// Few rows (at most 192) take one kernel, routed_small (see there).  More take these
 // launches, none of which needs a host round trip:
 //   role_count    per 1024-row chunk: its Nexus rows (only above 131,072 rows;
 //                 role_order counts for itself below);
@@ -520,13 +520,13 @@ routed_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
 
 // ------------------------------------------------------------- few rows
 //
-// T <= 192 rows: a generation step's projections, or a short turn's.  The call is
+// T <= 192 rows (see small_rows): a generation step's projections, or a short turn's.  The call is
 // bound by streaming the weights (4096 -> 6144: 50 MB), so the weights are the M
 // operand: a cluster of S CTAs takes 128 weight rows, each CTA a share of the
 // reduction, and NT >= T rows of X (unordered: no partition, no copy) are the N
-// operand.  S is the largest that keeps all clusters resident at once, so nearly
-// every SM streams its own share of the weights and no tile waits for a second
-// wave.  Both weight matrices are streamed where the rows hold both kinds, each
+// operand.  S is the largest that keeps all clusters resident at once, so no tile
+// waits for a second wave (48 weight tiles take S = 2, 96 of 152 SMs: of clusters of
+// three only 46 fit).  Both weight matrices are streamed where the rows hold both kinds, each
 // into an accumulator of its own, and the epilogue picks by role; with one kind
 // only, the other matrix is not read.  The partial sums (fp32) meet through
 // distributed shared memory in rank order.
