@@ -322,8 +322,9 @@ typedef struct {
  * a sequence cut between blocks leaves a partial (max, sum, accumulator) of
  * each piece in the workspace, and a second kernel merges them by log-sum-exp
  * (a sequence within one share is written directly).  With chunk_len > 0 (or
- * more than 1024 sequences, or a number of KV heads that suits the SMs badly)
- * the keys are split into chunks instead, whose (layer, sequence, KV head,
+ * more than 1024 sequences, or a number of KV heads that suits the SMs badly, or
+ * many or short sequences under more than 8 query heads per KV head) the keys are
+ * split into chunks instead, whose (layer, sequence, KV head,
  * chunk) units the blocks claim from a counter in the workspace (zeroed on
  * `stream` before the launch).  The workspace is never empty, and concurrent
  * calls need workspaces of their own.  A sequence whose rows fall outside [0, total_kv_rows) is

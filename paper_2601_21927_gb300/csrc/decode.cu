@@ -6,7 +6,8 @@
 //
 // Split-K, HBM-bound design:
 //   decode_tc      persistent blocks (one per SM) take equal shares of the keys
-//                  (or, for an explicit split, claim key chunks from a counter)
+//                  (or, for an explicit split and some short calls, claim key chunks
+//                  from a counter)
 //                  and stream their K/V tiles of 128 keys through a TMA ring; both contractions run
 //                  on the tensor cores with the keys in the M dimension (see
 //                  the kernel's comment); a single-chunk sequence writes O
@@ -71,7 +72,7 @@ __device__ __forceinline__ bool seq_refused(const DecParams &p, int raw_len, int
 // a counter to clear first (16 x 641 rows: 24.5, now 17.2; 64 long ragged ones, four layers,
 // 5.0 GB: 758, now 684-695, 7.2-7.4 TB/s).  The explicit split (chunk_len) and batches above kSeqCache
 // sequences, or KV heads that leave over an eighth of the SMs without a group, keep the
-// chunks.
+// chunks, and so do short or many sequences under many query heads (see make_plan).
 constexpr int kMinShare = 64;
 constexpr int kSnap = 32;
 
